@@ -21,7 +21,7 @@ struct es_plan {
   es_dtype_t dtype;
   int nseg;
   uint64_t numel;
-  uint64_t total_tiles;
+  uint64_t granules;
   esopt::SegDesc* d_segs;    // one allocation: the table, then (FP8) the
   float* d_inv_scale;        // reciprocal scales, or NULL
 };
@@ -70,7 +70,7 @@ es_status_t check_device_buffer(const void* p, const char* what) {
 }
 
 esopt::PlanView view(const es_plan* plan) {
-  return esopt::PlanView{plan->d_segs, plan->total_tiles, plan->dtype, plan->d_inv_scale};
+  return esopt::PlanView{plan->d_segs, plan->nseg, plan->granules, plan->dtype, plan->d_inv_scale};
 }
 
 es_status_t check_update_inputs(es_plan_t plan, const uint64_t* seeds, const float* coeffs, int n,
@@ -201,13 +201,12 @@ es_status_t create_plan(const es_segment_t* segs, const float* scales, int nseg,
       return fail(ES_ERR_OVERLAP, "segments %d and %d overlap in memory", order[k], order[k + 1]);
   }
 
-  const uint64_t tile = esopt::tile_elems(dtype);
-  uint64_t tiles = 0;
+  uint64_t granules = 0;
   for (int k = 0; k < nseg; ++k) {
-    table[k] = esopt::SegDesc{segs[k].data, segs[k].numel, segs[k].index_base, tiles};
-    tiles += (segs[k].numel + tile - 1) / tile;
+    table[k] = esopt::SegDesc{segs[k].data, segs[k].numel, segs[k].index_base, granules};
+    granules += esopt::granules_of(segs[k].numel);
   }
-  table[nseg] = esopt::SegDesc{nullptr, 0, 0, tiles};
+  table[nseg] = esopt::SegDesc{nullptr, 0, 0, granules};
 
   int device = -1;
   cudaError_t err = cudaGetDevice(&device);
@@ -252,7 +251,7 @@ es_status_t create_plan(const es_segment_t* segs, const float* scales, int nseg,
   plan->dtype = dtype;
   plan->nseg = nseg;
   plan->numel = total;
-  plan->total_tiles = tiles;
+  plan->granules = granules;
   *out = plan;
   return ok();
 }

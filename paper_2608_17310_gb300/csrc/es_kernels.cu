@@ -1,12 +1,12 @@
 // sm_103a kernels of the ES step: in-place perturb/restore (theta += s eps) and
 // the fused N-seed update (theta += sum_i c_i eps_i), plus a noise fill.
 //
-// All three stream the parameter set once per launch. Work is cut into tiles
-// of kBlockThreads threads x kVecsPerThread 16-byte vectors that never
-// straddle a segment; persistent CTAs walk the tiles in grid-stride
-// order, so consecutive CTAs touch consecutive memory and each CTA advances
-// through the segment table monotonically (one table lookup per tile, no
-// per-element search).
+// Both stream the parameter set once per launch. A plan's segments lie end to
+// end in a space of 16-element granules; a launch cuts that space into one
+// contiguous range per CTA, all of one length, with one large CTA per SM. A CTA
+// finds its first segment by a search and walks its range from there, so every
+// SM gets the same work whatever the set's size and however it is divided into
+// tensors.
 // Every element is owned by exactly one thread: no atomics, no shared state
 // between threads except the staged seeds of the update.
 #include <cuda_bf16.h>
@@ -28,6 +28,7 @@ struct Bf16Io {
   static constexpr int kVec = 8;
   static constexpr bool kScaled = false;
   using Scalar = uint16_t;
+  using Raw = uint4;  // a unit of 8 elements as stored
   __device__ static uint32_t pack2(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);  // one cvt.rn.bf16x2.f32
     return *reinterpret_cast<uint32_t*>(&h);
@@ -53,20 +54,28 @@ struct Bf16Io {
       f[k + 1] = hi(w);
     }
   }
-  // The first `rem` (< 8) elements at base[e], the rest zero, as one vector.
-  __device__ static uint4 load_partial(const uint16_t* base, uint64_t e, int rem) {
+  // The first `rem` (1 .. 8) elements of the unit at p, the rest zero.
+  __device__ static Raw load_unit(const uint16_t* p, int rem) {
+    if (rem == kUnit) return *reinterpret_cast<const uint4*>(p);
     uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < rem) w[k >> 1] |= static_cast<uint32_t>(base[e + k]) << (16 * (k & 1));
+    for (int k = 0; k < kUnit; ++k)
+      if (k < rem) w[k >> 1] |= static_cast<uint32_t>(p[k]) << (16 * (k & 1));
     return make_uint4(w[0], w[1], w[2], w[3]);
   }
-  __device__ static void store_partial(uint16_t* base, uint64_t e, int rem, const uint4& v) {
+  __device__ static void store_unit(uint16_t* p, int rem, const Raw& v) {
+    if (rem == kUnit) {
+      *reinterpret_cast<uint4*>(p) = v;
+      return;
+    }
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < rem) base[e + k] = static_cast<uint16_t>(w[k >> 1] >> (16 * (k & 1)));
+    for (int k = 0; k < kUnit; ++k)
+      if (k < rem) p[k] = static_cast<uint16_t>(w[k >> 1] >> (16 * (k & 1)));
   }
+  __device__ static Raw zero_unit() { return make_uint4(0u, 0u, 0u, 0u); }
+  __device__ static void unpack_unit(const Raw& v, float (&f)[kUnit]) { unpack(v, f); }
+  __device__ static Raw pack_unit(const float (&f)[kUnit]) { return pack(f); }
 };
 
 struct F32Io {
@@ -83,18 +92,45 @@ struct F32Io {
   }
   template <int M>
   __device__ static void round_trip(float (&)[M]) {}
-  __device__ static uint4 load_partial(const float* base, uint64_t e, int rem) {
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
+  struct Raw {
+    uint4 lo, hi;
+  };
+  __device__ static Raw load_unit(const float* p, int rem) {
+    if (rem == kUnit) {
+      const uint4* q = reinterpret_cast<const uint4*>(p);
+      return Raw{q[0], q[1]};
+    }
+    float f[kUnit];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (k < rem) w[k] = __float_as_uint(base[e + k]);
-    return make_uint4(w[0], w[1], w[2], w[3]);
+    for (int k = 0; k < kUnit; ++k) f[k] = k < rem ? p[k] : 0.0f;
+    return pack_unit(f);
   }
-  __device__ static void store_partial(float* base, uint64_t e, int rem, const uint4& v) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  __device__ static void store_unit(float* p, int rem, const Raw& v) {
+    if (rem == kUnit) {
+      uint4* q = reinterpret_cast<uint4*>(p);
+      q[0] = v.lo;
+      q[1] = v.hi;
+      return;
+    }
+    float f[kUnit];
+    unpack_unit(v, f);
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (k < rem) base[e + k] = __uint_as_float(w[k]);
+    for (int k = 0; k < kUnit; ++k)
+      if (k < rem) p[k] = f[k];
+  }
+  __device__ static Raw zero_unit() {
+    return Raw{make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+  }
+  __device__ static void unpack_unit(const Raw& v, float (&f)[kUnit]) {
+    const uint32_t w[kUnit] = {v.lo.x, v.lo.y, v.lo.z, v.lo.w, v.hi.x, v.hi.y, v.hi.z, v.hi.w};
+#pragma unroll
+    for (int k = 0; k < kUnit; ++k) f[k] = __uint_as_float(w[k]);
+  }
+  __device__ static Raw pack_unit(const float (&f)[kUnit]) {
+    return Raw{make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]),
+                          __float_as_uint(f[3])),
+               make_uint4(__float_as_uint(f[4]), __float_as_uint(f[5]), __float_as_uint(f[6]),
+                          __float_as_uint(f[7]))};
   }
 };
 
@@ -140,29 +176,39 @@ struct Fp8Io {
       f[k + 1] = r.y;
     }
   }
-  // The first `rem` (< 16) elements at base[e], the rest zero, as one vector.
-  __device__ static uint4 load_partial(const uint8_t* base, uint64_t e, int rem) {
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
+  using Raw = uint2;
+  __device__ static Raw load_unit(const uint8_t* p, int rem) {
+    if (rem == kUnit) return *reinterpret_cast<const uint2*>(p);
+    uint32_t w[2] = {0u, 0u};
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
-      if (k < rem) w[k >> 2] |= static_cast<uint32_t>(base[e + k]) << (8 * (k & 3));
-    return make_uint4(w[0], w[1], w[2], w[3]);
+    for (int k = 0; k < kUnit; ++k)
+      if (k < rem) w[k >> 2] |= static_cast<uint32_t>(p[k]) << (8 * (k & 3));
+    return make_uint2(w[0], w[1]);
   }
-  __device__ static void store_partial(uint8_t* base, uint64_t e, int rem, const uint4& v) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  __device__ static void store_unit(uint8_t* p, int rem, const Raw& v) {
+    if (rem == kUnit) {
+      *reinterpret_cast<uint2*>(p) = v;
+      return;
+    }
+    const uint32_t w[2] = {v.x, v.y};
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
-      if (k < rem) base[e + k] = static_cast<uint8_t>(w[k >> 2] >> (8 * (k & 3)));
+    for (int k = 0; k < kUnit; ++k)
+      if (k < rem) p[k] = static_cast<uint8_t>(w[k >> 2] >> (8 * (k & 3)));
+  }
+  __device__ static Raw zero_unit() { return make_uint2(0u, 0u); }
+  __device__ static void unpack_unit(const Raw& v, float (&f)[kUnit]) {
+    const uint32_t w[2] = {v.x, v.y};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float2 a = dec2(w[k]), b = dec2(w[k] >> 16);
+      f[4 * k + 0] = a.x; f[4 * k + 1] = a.y; f[4 * k + 2] = b.x; f[4 * k + 3] = b.y;
+    }
+  }
+  __device__ static Raw pack_unit(const float (&f)[kUnit]) {
+    return make_uint2(enc2(f[0], f[1]) | (enc2(f[2], f[3]) << 16),
+                      enc2(f[4], f[5]) | (enc2(f[6], f[7]) << 16));
   }
 };
-
-// Vectors a thread processes at once for a kernel kind's group g (g bf16
-// vectors of 8 elements): the same number of elements, hence of Philox
-// chains, for every storage type, within the kVecsPerThread vectors of a tile.
-template <class Io>
-__host__ __device__ constexpr int group_for(int g) {
-  return Io::kVec > 8 ? (g > 1 ? g / 2 : 1) : Io::kVec < 8 ? (2 * g < kVecsPerThread ? 2 * g : kVecsPerThread) : g;
-}
 
 // theta + acc in storage units: acc is in parameter units, so a scaled
 // segment takes acc / scale (one fused multiply-add with 1 / scale).
@@ -172,403 +218,342 @@ __device__ __forceinline__ float add_acc(float theta, float acc, float inv_scale
   else return theta + acc;
 }
 
-// Philox words of block j for one seed. SchedGen serves the blocks of a tile
-// that share the high counter word, with the round keys read from a
-// precomputed schedule (kernel parameters or registers loaded from shared
-// memory) and the tile's constants computed once; AnyGen serves any block. Both
-// give the same words.
+// Philox words of one seed's blocks that share the high counter word, with the
+// round keys read from a precomputed schedule (kernel parameters, or registers
+// loaded from shared memory) and the constants of that word given.
 template <class Keys, bool kWideFirst = false>
 struct SchedGen {
   TileConst t;
   uint32_t rk1, rk2;  // round 0's k1, round 1's k0
   Keys rk;            // rounds 2..9: rk[2r - 4], rk[2r - 3]
-  __device__ uint4 block(uint64_t j) const {
-    return philox_block_rk<kWideFirst>(static_cast<uint32_t>(j), t, rk1, rk2, rk);
-  }
-  // The same words from round 0's product (philox_round0 of the block's j_lo).
+  // From round 0's product (philox_round0 of the block's low counter word).
   __device__ uint4 block_r0(Round0 p0) const {
     return philox_block_r0<kWideFirst>(p0, t, rk1, rk2, rk);
   }
 };
-struct AnyGen {
-  PhiloxKey key;
-  __device__ uint4 block(uint64_t j) const { return philox_block(j, key); }
-};
 
 // Generator of one seed whose schedule is a kernel parameter.
-template <bool kUniformHi, bool kWideFirst = false>
-__device__ __forceinline__ auto sched_gen(const PhiloxSched& s, uint32_t j_hi) {
-  if constexpr (kUniformHi)
-    return SchedGen<const uint32_t*, kWideFirst>{tile_const(j_hi, s.rk[0], s.rk[3]), s.rk[1],
-                                                 s.rk[2], s.rk + 4};
-  else return AnyGen{PhiloxKey{s.rk[0], s.rk[1]}};
+template <bool kWideFirst>
+__device__ __forceinline__ SchedGen<const uint32_t*, kWideFirst> sched_gen(const PhiloxSched& s,
+                                                                          uint32_t j_hi) {
+  return {tile_const(j_hi, s.rk[0], s.rk[3]), s.rk[1], s.rk[2], s.rk + 4};
 }
 
-// How each Philox block becomes theta updates. The forms give bit-identical
-// values: a packed two-wide FP32 instruction rounds each half exactly like the
-// scalar one. They differ only in instruction mix, which moves work between the
-// FMA pipe's halves. Each kernel uses the form measured fastest for it:
-//   kScalar     scalar transform (polar) and scalar FMAs;
-//   kPackedFma  scalar transform, packed FMAs into theta or the accumulator;
-//   kPacked     packed transform (polar2) and packed FMAs.
-enum class NoiseForm { kScalar, kPackedFma, kPacked };
-constexpr NoiseForm kAxpy1Form = static_cast<NoiseForm>(ES_AXPY1_FORM);
-constexpr NoiseForm kAxpy2Form = static_cast<NoiseForm>(ES_AXPY2_FORM);
-constexpr NoiseForm kUpdateForm = static_cast<NoiseForm>(ES_UPDATE_FORM);
-constexpr bool kUpdatePipelined = ES_UPDATE_PIPELINED != 0;
-constexpr bool kUpdatePingPong = ES_UPDATE_PIPELINED >= 2;
-constexpr int kRound0 = ES_ROUND0;
-constexpr bool kFlipPacked = ES_FLIP_PACKED != 0;
-// Near-one radius inputs: a rare branch (true) or a select per pair (false).
-constexpr bool kNearOneBranch = ES_NEAR_ONE_BRANCH != 0;
-
-// The radius of every pair, from its radius^2.
+// The pairs of NB Philox blocks in polar form (r, cos, sin) from their words,
+// with packed two-wide FP32 instructions (each half rounds exactly like the
+// scalar instruction) and the near-one radius inputs on a rare branch.
 template <int NB>
-__device__ __forceinline__ void polar_roots(Polar2 (&p)[NB]) {
-#pragma unroll
-  for (int b = 0; b < NB; ++b) p[b].r = make_float2(sqrt_approx(p[b].r.x), sqrt_approx(p[b].r.y));
-}
-
-// The pairs of NB Philox blocks in polar form (r, cos, sin) from their words.
-template <NoiseForm kForm, int NB>
 __device__ __forceinline__ void polar_from_words(const uint4 (&x)[NB], Polar2 (&p)[NB]) {
-  constexpr bool kLogOnly = kNearOneBranch;
   uint2 xa[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     xa[b] = make_uint2(x[b].x, x[b].z);
-    if constexpr (kForm == NoiseForm::kPacked) {
-      p[b] = polar2_sq<kLogOnly>(x[b]);
-    } else {
-      const Polar a = polar_sq<kLogOnly>(x[b].x, x[b].y), c = polar_sq<kLogOnly>(x[b].z, x[b].w);
-      p[b] = Polar2{make_float2(a.r, c.r), make_float2(a.c, c.c), make_float2(a.s, c.s)};
-    }
+    p[b] = polar2_sq<true>(x[b]);
   }
-  if constexpr (kLogOnly) fix_near_one<NB>(xa, p);
-  polar_roots<NB>(p);
-}
-
-// Words of Philox blocks j0 .. j0 + NB - 1.
-template <int NB, class Gen>
-__device__ __forceinline__ void philox_words(const Gen& gen, uint64_t j0, uint4 (&x)[NB]) {
+  fix_near_one<NB>(xa, p);
 #pragma unroll
-  for (int b = 0; b < NB; ++b) x[b] = gen.block(j0 + b);
-}
-
-template <NoiseForm kForm, int NB, class Gen>
-__device__ __forceinline__ void polar_blocks(const Gen& gen, uint64_t j0, Polar2 (&p)[NB]) {
-  uint4 x[NB];
-  philox_words<NB>(gen, j0, x);
-  polar_from_words<kForm, NB>(x, p);
+  for (int b = 0; b < NB; ++b) p[b].r = make_float2(sqrt_approx(p[b].r.x), sqrt_approx(p[b].r.y));
 }
 
 // f[k] += scale * eps[4 j0 + k] for the V elements of blocks whose polar
-// forms are pp[0 .. V / 4), with scale folded into each pair's radius.
-template <NoiseForm kForm, int V>
-__device__ __forceinline__ void apply_noise(const Polar2* pp, float scale, float (&f)[V]) {
-  constexpr int NB = V / 4;
+// forms are pp, with scale folded into each pair's radius.
+template <int V>
+__device__ __forceinline__ void apply_noise(const Polar2 (&pp)[V / 4], float scale, float (&f)[V]) {
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {
+  for (int b = 0; b < V / 4; ++b) {
     const Polar2& p = pp[b];
-    if constexpr (kForm == NoiseForm::kScalar) {
-      const float sp = -(scale * p.r.x), sq = -(scale * p.r.y);
-      f[4 * b + 0] = fmaf(sp, p.c.x, f[4 * b + 0]);
-      f[4 * b + 1] = fmaf(sp, p.s.x, f[4 * b + 1]);
-      f[4 * b + 2] = fmaf(sq, p.c.y, f[4 * b + 2]);
-      f[4 * b + 3] = fmaf(sq, p.s.y, f[4 * b + 3]);
-    } else {
-      const float2 sr = __fmul2_rn(make_float2(-scale, -scale), p.r);   // -(scale * r)
-      const float2 lo = __ffma2_rn(make_float2(sr.x, sr.x), make_float2(p.c.x, p.s.x),
-                                   make_float2(f[4 * b + 0], f[4 * b + 1]));
-      const float2 hi = __ffma2_rn(make_float2(sr.y, sr.y), make_float2(p.c.y, p.s.y),
-                                   make_float2(f[4 * b + 2], f[4 * b + 3]));
-      f[4 * b + 0] = lo.x;
-      f[4 * b + 1] = lo.y;
-      f[4 * b + 2] = hi.x;
-      f[4 * b + 3] = hi.y;
-    }
+    const float2 sr = __fmul2_rn(make_float2(-scale, -scale), p.r);   // -(scale * r)
+    const float2 lo = __ffma2_rn(make_float2(sr.x, sr.x), make_float2(p.c.x, p.s.x),
+                                 make_float2(f[4 * b + 0], f[4 * b + 1]));
+    const float2 hi = __ffma2_rn(make_float2(sr.y, sr.y), make_float2(p.c.y, p.s.y),
+                                 make_float2(f[4 * b + 2], f[4 * b + 3]));
+    f[4 * b + 0] = lo.x;
+    f[4 * b + 1] = lo.y;
+    f[4 * b + 2] = hi.x;
+    f[4 * b + 3] = hi.y;
   }
-}
-
-// f[k] += scale * eps[4 j0 + k] for the V elements of Philox blocks j0,
-// j0 + 1, ..., with scale folded into each pair's radius.
-template <NoiseForm kForm, int V, class Gen>
-__device__ __forceinline__ void add_scaled_noise(const Gen& gen, uint64_t j0, float scale,
-                                                 float (&f)[V]) {
-  Polar2 pp[V / 4];
-  polar_blocks<kForm, V / 4>(gen, j0, pp);
-  apply_noise<kForm, V>(pp, scale, f);
 }
 
 // f[k] += scale * eps for the V elements of the Philox blocks whose words
 // are x.
-template <NoiseForm kForm, int V>
-__device__ __forceinline__ void add_scaled_noise_words(const uint4 (&x)[V / 4], float scale,
-                                                       float (&f)[V]) {
+template <int V>
+__device__ __forceinline__ void add_scaled_noise(const uint4 (&x)[V / 4], float scale,
+                                                 float (&f)[V]) {
   Polar2 pp[V / 4];
-  polar_from_words<kForm, V / 4>(x, pp);
-  apply_noise<kForm, V>(pp, scale, f);
+  polar_from_words<V / 4>(x, pp);
+  apply_noise<V>(pp, scale, f);
 }
 
-// f <- round(round(f + s1 * eps) + s2 * eps) for one seed's noise, computed
-// once: an antithetic restore (+eps out) followed by the perturb (-eps in).
-template <class Io, int V, class Gen>
-__device__ __forceinline__ void add_scaled_noise_twice(const Gen& gen, uint64_t j0, float s1,
-                                                       float s2, float (&f)[V]) {
-  constexpr int NB = V / 4;
-  Polar2 pp[NB];
-  polar_blocks<NoiseForm::kScalar, NB>(gen, j0, pp);
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const Polar2& p = pp[b];
-    float h[4];
-    h[0] = fmaf(-(s1 * p.r.x), p.c.x, f[4 * b + 0]);
-    h[1] = fmaf(-(s1 * p.r.x), p.s.x, f[4 * b + 1]);
-    h[2] = fmaf(-(s1 * p.r.y), p.c.y, f[4 * b + 2]);
-    h[3] = fmaf(-(s1 * p.r.y), p.s.y, f[4 * b + 3]);
-    Io::round_trip(h);
-    f[4 * b + 0] = fmaf(-(s2 * p.r.x), p.c.x, h[0]);
-    f[4 * b + 1] = fmaf(-(s2 * p.r.x), p.s.x, h[1]);
-    f[4 * b + 2] = fmaf(-(s2 * p.r.y), p.c.y, h[2]);
-    f[4 * b + 3] = fmaf(-(s2 * p.r.y), p.s.y, h[3]);
+// Segment of `granule`, at or after `lo` (segs[lo].granule_begin <= granule):
+// the warp tests 32 evenly spaced entries at a time, one per lane, so a table
+// of n segments takes log32(n) dependent loads. The loads are L2 latency and
+// nothing else: on a set of 200 ragged tensors a walk from entry 0 was most of a
+// launch (40 us of which a search leaves 5). Called by whole warps; every lane
+// returns the same segment.
+__device__ __forceinline__ int search_segment(const SegDesc* __restrict__ segs, int lo, int nseg,
+                                              uint64_t granule) {
+  const int lane = static_cast<int>(threadIdx.x & 31u);
+  int hi = nseg;  // granule < segs[hi].granule_begin
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) / 32;
+    const int probe = lo + step * (lane + 1);
+    const bool passed = probe < hi && segs[probe].granule_begin <= granule;
+    const int c = __popc(__ballot_sync(0xFFFFFFFFu, passed));  // a prefix of the lanes
+    lo += step * c;
+    hi = lo + step < hi ? lo + step : hi;
   }
+  return lo;
 }
 
-// Segment of `tile`; `seg` is the CTA's cursor and only moves forward.
-__device__ __forceinline__ const SegDesc* find_segment(const SegDesc* __restrict__ segs,
-                                                       int& seg, uint64_t tile) {
-  while (tile >= segs[seg + 1].tile_begin) ++seg;
-  return segs + seg;
+// The same among segments lo .. hi by one thread alone (bisection).
+__device__ __forceinline__ int segment_between(const SegDesc* __restrict__ segs, int lo, int hi,
+                                               uint64_t granule) {
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (segs[mid].granule_begin <= granule) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
 }
 
-// Whether every global index of the tile's elements [t0, t0 + tile) (clipped
-// to the segment) shares the high word of its Philox block counter, i.e. the
-// tile does not cross a multiple of 2^34 in index space.
-__device__ __forceinline__ bool uniform_hi(uint64_t index_base, uint64_t t0, uint64_t tile,
-                                           uint64_t numel) {
-  const uint64_t last = index_base + (t0 + tile < numel ? t0 + tile : numel) - 1;
-  return ((index_base + t0) >> 34) == (last >> 34);
+// A launch's division of the plan: `granules` in ranges of `per_cta`, the last
+// one shorter. The host makes the grid so that no range is empty.
+struct Split {
+  uint64_t granules;
+  uint64_t per_cta;
+};
+constexpr int kUnitsPerGranule = kGranule / kUnit;
+
+__device__ __forceinline__ uint64_t range_begin(const Split& s) { return blockIdx.x * s.per_cta; }
+__device__ __forceinline__ uint64_t range_end(const Split& s) {
+  const uint64_t e = range_begin(s) + s.per_cta;
+  return e < s.granules ? e : s.granules;
 }
 
-// Location of one tile: its segment's storage, the tile's first element and,
-// for a scaled storage type, 1 / the segment's scale.
+// The unit of 8 elements that a thread takes from a range: `rem` of them lie in
+// the segment (0: none).
 template <class Io>
-struct TileRef {
-  typename Io::Scalar* base;
-  uint64_t numel;
-  uint64_t index_base;
-  uint64_t t0;
-  float inv;
+struct UnitRef {
+  typename Io::Scalar* p;
+  int rem;
+  uint64_t j0;  // Philox block of element 0 (index bases are multiples of 8)
+  float inv;    // 1 / the segment's scale, for a scaled storage type
 };
 
 template <class Io>
-__device__ __forceinline__ TileRef<Io> tile_ref(const SegDesc* __restrict__ segs,
-                                                const float* __restrict__ inv_scale, int& seg,
-                                                uint64_t tile) {
-  constexpr uint64_t kTile = static_cast<uint64_t>(kBlockThreads) * kVecsPerThread * Io::kVec;
-  const SegDesc* d = find_segment(segs, seg, tile);
-  return TileRef<Io>{static_cast<typename Io::Scalar*>(d->data), d->numel, d->index_base,
-                     (tile - d->tile_begin) * kTile, Io::kScaled ? inv_scale[seg] : 1.0f};
+__device__ __forceinline__ UnitRef<Io> unit_ref(const SegDesc* __restrict__ segs,
+                                                const float* __restrict__ inv_scale, int seg,
+                                                uint64_t unit) {
+  const SegDesc d = segs[seg];
+  const uint64_t e = (unit - d.granule_begin * kUnitsPerGranule) * kUnit;
+  UnitRef<Io> r;
+  r.rem = e >= d.numel ? 0 : d.numel - e < kUnit ? static_cast<int>(d.numel - e) : kUnit;
+  r.p = static_cast<typename Io::Scalar*>(d.data) + e;
+  r.j0 = (d.index_base + e) >> 2;
+  r.inv = Io::kScaled ? inv_scale[seg] : 1.0f;
+  return r;
 }
 
-// First element of the calling thread's vector u of a tile. Vector u of a
-// tile is 256 consecutive 16-byte vectors, one per thread: each load and
-// store instruction of a warp covers 512 contiguous bytes.
-template <class Io>
-__device__ __forceinline__ uint64_t vec_elem(const TileRef<Io>& r, int u) {
-  return r.t0 + static_cast<uint64_t>(u * kBlockThreads + threadIdx.x) * Io::kVec;
-}
-
-// Vectors u0 .. u0 + G - 1 of the calling thread: a 16-byte load each; the
-// ragged end of a segment element by element, zeros past it.
-template <class Io, int G>
-__device__ __forceinline__ void load_group(const TileRef<Io>& r, int u0, uint4 (&v)[G]) {
-#pragma unroll
-  for (int q = 0; q < G; ++q) {
-    const uint64_t e = vec_elem(r, u0 + q);
-    v[q] = make_uint4(0u, 0u, 0u, 0u);
-    if (e + Io::kVec <= r.numel)
-      v[q] = *reinterpret_cast<const uint4*>(r.base + e);
-    else if (e < r.numel)
-      v[q] = Io::load_partial(r.base, e, static_cast<int>(r.numel - e));
-  }
-}
-
-template <class Io>
-__device__ __forceinline__ void store_vec(const TileRef<Io>& r, uint64_t e, const uint4& v) {
-  if (e + Io::kVec <= r.numel)
-    *reinterpret_cast<uint4*>(r.base + e) = v;
-  else if (e < r.numel)
-    Io::store_partial(r.base, e, static_cast<int>(r.numel - e), v);
-}
+// What a pass over the parameters does: one step theta += scale1 * eps_seed1;
+// two steps, the second on the first's result rounded to the storage type
+// (restore of one member fused with the perturb of the next); or the two steps
+// of one seed, whose noise is generated once (the antithetic flip).
+enum class AxpyMode { kOne, kTwo, kFlip };
 
 // Arguments of a perturb/restore launch: the schedule and scale of each step
-// (step 2 only with kTwo). A __grid_constant__ parameter, so every round key
+// (step 2 unused by kOne). A __grid_constant__ parameter, so every round key
 // is read from the constant bank as an instruction operand.
 struct AxpyArgs {
   PhiloxSched s1, s2;
   float scale1, scale2;
 };
 
-// One tile of the perturb/restore pass (kTwo: fused restore + perturb; kSame:
-// both steps use one seed, whose noise is generated once), G vectors at a
-// time. The loads of the next group (at the last group: the first group of
-// the CTA's next tile, `next`) are issued before the current group is
-// computed, so the memory latency hides behind the generator's work. kFull:
-// the whole tile lies inside its segment (every tile but a segment's last),
-// so its vectors are addressed from one per-thread pointer and block index
-// without bounds checks.
-template <class Io, bool kTwo, bool kSame, bool kUniformHi, bool kFull, int G>
-__device__ __forceinline__ void axpy_tile(const TileRef<Io>& cur, uint4 (&v)[G],
-                                          const AxpyArgs& a, const SegDesc* __restrict__ segs,
-                                          const float* __restrict__ inv_scale, int& seg,
-                                          uint64_t next, bool has_next, TileRef<Io>& nxt) {
-  constexpr int V = Io::kVec;
-  constexpr NoiseForm kAxpyForm = kTwo ? kAxpy2Form : kAxpy1Form;
-  constexpr int kGroups = kVecsPerThread / G;
-  constexpr int kStride = kBlockThreads * V;  // elements from one vector of a thread to the next
-  const uint32_t j_hi = static_cast<uint32_t>((cur.index_base + cur.t0) >> 34);
-  // the one-seed pass is fastest with every Philox product 64-bit wide (in
-  // FP8 storage, with twice the blocks per vector, that spills)
-  constexpr bool kWide1 = !kTwo && V <= 8;
-  const auto gen = sched_gen<kUniformHi, kWide1>(a.s1, j_hi);
-  const auto gen2 = sched_gen<kUniformHi && kTwo && !kSame>(a.s2, j_hi);
-  const float s1 = a.scale1 * cur.inv, s2 = a.scale2 * cur.inv;
-  // the thread's first element of the tile, and its Philox block (index_base
-  // is a multiple of 8 and t0 of the tile size, so the division is exact)
-  typename Io::Scalar* const p = cur.base + cur.t0 + threadIdx.x * V;
-  const uint64_t j_thread = ((cur.index_base + cur.t0) >> 2) + threadIdx.x * (V / 4);
-  // Round 0's product from the counter alone (kRound0): once per block for
-  // both seeds of the fused pass, and in a tile inside its segment stepped
-  // from the thread's first block (its blocks share the high counter word,
-  // so j_lo + d never wraps).
-  constexpr int NB = V / 4;
-  constexpr bool kR0 = kUniformHi && (kSame ? kFlipPacked && kFull && kRound0 >= 2
-                                            : (kRound0 >= 2 ? (kFull || kTwo)
-                                                            : kRound0 >= 1 && kTwo));
-  constexpr bool kR0Step = kR0 && kFull && kRound0 >= 2;
-  Round0 p0_thread{0u, 0u};
-  if constexpr (kR0Step) p0_thread = philox_round0<kWide1>(static_cast<uint32_t>(j_thread));
-#pragma unroll
-  for (int grp = 0; grp < kGroups; ++grp) {
-    uint4 nv[G];
-    if (grp + 1 < kGroups) {
-      if constexpr (kFull) {
-#pragma unroll
-        for (int q = 0; q < G; ++q)
-          nv[q] = *reinterpret_cast<const uint4*>(p + ((grp + 1) * G + q) * kStride);
-      } else {
-        load_group<Io, G>(cur, (grp + 1) * G, nv);
-      }
-    } else if (has_next) {
-      nxt = tile_ref<Io>(segs, inv_scale, seg, next);
-      load_group<Io, G>(nxt, 0, nv);
-    }
-#pragma unroll
-    for (int q = 0; q < G; ++q) {
-      const int u = grp * G + q;
-      if constexpr (!kFull) {
-        if (vec_elem(cur, u) >= cur.numel) continue;
-      }
-      const uint64_t j0 = j_thread + static_cast<uint64_t>(u) * (kStride / 4);
-      float f[V];
-      Io::unpack(v[q], f);
-      if constexpr (kSame && kFlipPacked) {
-        // one seed's noise for both steps, in the packed form
-        uint4 x[NB];
-        if constexpr (kR0) {
-#pragma unroll
-          for (int b = 0; b < NB; ++b)
-            x[b] = gen.block_r0(
-                round0_step(p0_thread, static_cast<uint32_t>(u * (kStride / 4) + b)));
-        } else {
-          philox_words<NB>(gen, j0, x);
-        }
-        Polar2 pp[NB];
-        polar_from_words<kAxpyForm, NB>(x, pp);
-        apply_noise<kAxpyForm, V>(pp, s1, f);
-        Io::round_trip(f);
-        apply_noise<kAxpyForm, V>(pp, s2, f);
-      } else if constexpr (kSame) {
-        add_scaled_noise_twice<Io, V>(gen, j0, s1, s2, f);
-      } else if constexpr (kR0) {
-        Round0 p0[NB];
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-          p0[b] = kR0Step ? round0_step(p0_thread, static_cast<uint32_t>(u * (kStride / 4) + b))
-                          : philox_round0<kWide1>(static_cast<uint32_t>(j0 + b));
-        uint4 x[NB];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) x[b] = gen.block_r0(p0[b]);
-        add_scaled_noise_words<kAxpyForm, V>(x, s1, f);
-        if constexpr (kTwo) {
-          Io::round_trip(f);
-#pragma unroll
-          for (int b = 0; b < NB; ++b) x[b] = gen2.block_r0(p0[b]);
-          add_scaled_noise_words<kAxpyForm, V>(x, s2, f);
-        }
-      } else {
-        add_scaled_noise<kAxpyForm, V>(gen, j0, s1, f);
-        if constexpr (kTwo) {
-          Io::round_trip(f);
-          add_scaled_noise<kAxpyForm, V>(gen2, j0, s2, f);
-        }
-      }
-      if constexpr (kFull)
-        *reinterpret_cast<uint4*>(p + u * kStride) = Io::pack(f);
-      else
-        store_vec(cur, vec_elem(cur, u), Io::pack(f));
-    }
-    if (grp + 1 < kGroups || has_next) {
-#pragma unroll
-      for (int q = 0; q < G; ++q) v[q] = nv[q];
+// The steps of kMode on the V values f. words(second, x) gives the Philox words
+// of the first or the second seed's blocks.
+template <class Io, AxpyMode kMode, int V, class Words>
+__device__ __forceinline__ void axpy_values(const Words& words, float s1, float s2, float (&f)[V]) {
+  uint4 x[V / 4];
+  words(false, x);
+  if constexpr (kMode == AxpyMode::kFlip) {
+    Polar2 pp[V / 4];
+    polar_from_words<V / 4>(x, pp);
+    apply_noise<V>(pp, s1, f);
+    Io::round_trip(f);
+    apply_noise<V>(pp, s2, f);
+  } else {
+    add_scaled_noise<V>(x, s1, f);
+    if constexpr (kMode == AxpyMode::kTwo) {
+      Io::round_trip(f);
+      words(true, x);
+      add_scaled_noise<V>(x, s2, f);
     }
   }
 }
 
-// theta[g] <- round(theta[g] + scale * eps_seed[g]) over every segment; with
-// kTwo, a second step round(. + scale2 * eps_seed2[g]) follows in registers,
-// after the first result has been rounded to the storage type exactly as a
-// separate launch would store it (restore of one member fused with the
-// perturb of the next).
-// For a scaled storage type (FP8) the noise is added in units of the
-// segment's scale: scale * inv_scale[segment].
-template <class Io, bool kTwo, bool kSame>
-__global__ void __launch_bounds__(kBlockThreads, axpy_min_blocks(kTwo, Io::kVec, kSame))
-axpy_noise_kernel(const SegDesc* __restrict__ segs, const float* __restrict__ inv_scale,
-                  uint64_t total_tiles, const __grid_constant__ AxpyArgs a) {
-  constexpr int G = group_for<Io>(kTwo ? kAxpy2Group : kAxpy1Group);
-  uint64_t tile = blockIdx.x;
-  if (tile >= total_tiles) return;
-  int seg = 0;
-  TileRef<Io> cur = tile_ref<Io>(segs, inv_scale, seg, tile);
-  uint4 v[G];
-  load_group<Io, G>(cur, 0, v);
+// Shape of a pass: threads of its one CTA per SM, 16-byte vectors per thread
+// in a tile (the unrolled body of the loop) and how many vectors ahead theta is
+// loaded. What bounds the passes is the generator's instruction stream: the
+// FMA-heavy pipe (integer products), MUFU and issue, and, seen by what moves
+// them, instruction fetch: all of an SM's warps in one CTA on a loop body of
+// 300-600 instructions run 6-15 % faster than 2 or 3 CTAs of 256 threads on one
+// of 1200. Measured on sm_103a over 792,680,960 parameters (us; 256 threads, 4
+// vectors, 1 ahead, grid-stride tiles -> this): bf16 one step 678 -> 569 (5.58 TB/s), two
+// steps 1217 -> 1094 (1.449e12 Gaussians/s), flip 729 -> 621; fp32 971 -> 962 (6.59 TB/s: HBM),
+// 1366 -> 1077, 976 -> 961; FP8 636 -> 575, 1301 -> 1127, 718 -> 639.
+// Thread counts that are no multiple of 128 leave the SM's four schedulers
+// unequal warps and run 10 % slower.
+struct AxpyShape {
+  int threads, vecs, ahead;
+};
+template <class Io, AxpyMode kMode>
+__host__ __device__ constexpr AxpyShape axpy_shape() {
+  if (Io::kVec == 4) return {1024, 4, 2};
+  if (Io::kVec == 16) return kMode == AxpyMode::kTwo ? AxpyShape{640, 2, 2} : AxpyShape{768, 2, 1};
+  return kMode == AxpyMode::kOne   ? AxpyShape{1024, 2, 2}
+         : kMode == AxpyMode::kTwo ? AxpyShape{1024, 2, 1}
+                                   : AxpyShape{1024, 3, 1};
+}
+// Units of one tile.
+template <class Io, AxpyMode kMode>
+__host__ __device__ constexpr uint64_t axpy_tile_units() {
+  constexpr AxpyShape k = axpy_shape<Io, kMode>();
+  return static_cast<uint64_t>(k.threads) * k.vecs * Io::kVec / kUnit;
+}
+
+// `tiles` whole tiles of one segment, all with the same high counter word,
+// from the calling thread's first vector at p, whose first Philox block is
+// j_thread. Vector u of a tile is one 16-byte vector per thread, so each load
+// and store instruction of a warp covers 512 contiguous bytes; the load of the
+// vector `ahead` of the current one is issued before that is computed. Round 0's Philox
+// product (of the counter alone) is stepped by 64-bit additions from the
+// thread's first block instead of multiplied.
+template <class Io, AxpyMode kMode>
+__device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thread, uint32_t tiles,
+                                         const AxpyArgs& a, float inv) {
+  constexpr int V = Io::kVec, NB = V / 4;
+  constexpr AxpyShape kShape = axpy_shape<Io, kMode>();
+  constexpr int D = kShape.ahead;
+  constexpr int kStride = kShape.threads * V;  // elements between a thread's vectors
+  static_assert(kShape.vecs % D == 0, "the vectors in flight rotate within a tile");
+  // the one-seed pass is fastest with every Philox product 64-bit wide (in
+  // FP8 storage, with twice the blocks per vector, that spills)
+  constexpr bool kWide = kMode == AxpyMode::kOne && V <= 8;
+  const uint32_t j_hi = static_cast<uint32_t>(j_thread >> 32);
+  const auto gen1 = sched_gen<kWide>(a.s1, j_hi);
+  const auto gen2 = sched_gen<kWide>(a.s2, j_hi);
+  const float s1 = a.scale1 * inv, s2 = a.scale2 * inv;
+  Round0 p0 = philox_round0<kWide>(static_cast<uint32_t>(j_thread));
+  uint4 v[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) v[k] = *reinterpret_cast<const uint4*>(p + k * kStride);
+#pragma unroll 1
   for (;;) {
-    const uint64_t next = tile + gridDim.x;
-    const bool has_next = next < total_tiles;
-    TileRef<Io> nxt = cur;
-    constexpr uint64_t kTile = static_cast<uint64_t>(kBlockThreads) * kVecsPerThread * Io::kVec;
-    if (!uniform_hi(cur.index_base, cur.t0, kTile, cur.numel))
-      axpy_tile<Io, kTwo, kSame, false, false, G>(cur, v, a, segs, inv_scale, seg, next, has_next,
-                                                  nxt);
-    else if (cur.t0 + kTile <= cur.numel)
-      axpy_tile<Io, kTwo, kSame, true, true, G>(cur, v, a, segs, inv_scale, seg, next, has_next,
-                                                nxt);
-    else
-      axpy_tile<Io, kTwo, kSame, true, false, G>(cur, v, a, segs, inv_scale, seg, next, has_next,
-                                                 nxt);
-    if (!has_next) break;
-    tile = next;
-    cur = nxt;
+#pragma unroll
+    for (int u = 0; u < kShape.vecs; ++u) {
+      float f[V];
+      Io::unpack(v[u % D], f);
+      if (u + D < kShape.vecs || tiles > 1)
+        v[u % D] = *reinterpret_cast<const uint4*>(p + (u + D) * kStride);
+      Round0 r0[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) r0[b] = round0_step(p0, static_cast<uint32_t>(u * (kStride / 4) + b));
+      axpy_values<Io, kMode, V>(
+          [&](bool second, uint4 (&x)[NB]) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b) x[b] = second ? gen2.block_r0(r0[b]) : gen1.block_r0(r0[b]);
+          },
+          s1, s2, f);
+      *reinterpret_cast<uint4*>(p + u * kStride) = Io::pack(f);
+    }
+    if (--tiles == 0) return;
+    p += kShape.vecs * kStride;
+    p0 = round0_step(p0, kShape.vecs * (kStride / 4));
+  }
+}
+
+// Units q .. stop - 1, which lie in segments first .. last: one unit per
+// thread at a time, its segment found by the thread itself.
+template <class Io, AxpyMode kMode>
+__device__ __forceinline__ void axpy_units(const SegDesc* __restrict__ segs,
+                                           const float* __restrict__ inv_scale, int first, int last,
+                                           uint64_t q, uint64_t stop, const AxpyArgs& a) {
+  constexpr int NB = kUnit / 4;
+#pragma unroll 1
+  for (q += threadIdx.x; q < stop; q += blockDim.x) {
+    const UnitRef<Io> r = unit_ref<Io>(
+        segs, inv_scale, segment_between(segs, first, last, q / kUnitsPerGranule), q);
+    if (r.rem == 0) continue;
+    const typename Io::Raw raw = Io::load_unit(r.p, r.rem);
+    float f[kUnit];
+    Io::unpack_unit(raw, f);
+    // a unit's two blocks start at an even one, so they share the high word
+    const uint32_t j_hi = static_cast<uint32_t>(r.j0 >> 32);
+    const auto gen1 = sched_gen<false>(a.s1, j_hi);
+    const auto gen2 = sched_gen<false>(a.s2, j_hi);
+    Round0 r0[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) r0[b] = philox_round0<false>(static_cast<uint32_t>(r.j0 + b));
+    axpy_values<Io, kMode, kUnit>(
+        [&](bool second, uint4 (&x)[NB]) {
+#pragma unroll
+          for (int b = 0; b < NB; ++b) x[b] = second ? gen2.block_r0(r0[b]) : gen1.block_r0(r0[b]);
+        },
+        a.scale1 * r.inv, a.scale2 * r.inv, f);
+    Io::store_unit(r.p, r.rem, Io::pack_unit(f));
+  }
+}
+
+// theta[g] <- round(theta[g] + scale * eps_seed[g]) over every segment, or the
+// two steps of kTwo and kFlip. For a scaled storage type (FP8) the noise is
+// added in units of the segment's scale: scale * inv_scale[segment].
+// A CTA alternates between runs of whole tiles inside one segment (axpy_run)
+// and up to a tile's worth of units wherever a segment, the range or a high
+// counter word ends (axpy_units).
+template <class Io, AxpyMode kMode>
+__global__ void __launch_bounds__(axpy_shape<Io, kMode>().threads, 1)
+axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
+                  const Split split, const __grid_constant__ AxpyArgs a) {
+  constexpr AxpyShape kShape = axpy_shape<Io, kMode>();
+  constexpr uint64_t kTile = axpy_tile_units<Io, kMode>();
+  uint64_t q = range_begin(split) * kUnitsPerGranule;
+  const uint64_t end = range_end(split) * kUnitsPerGranule;
+  int seg = search_segment(segs, 0, nseg, q / kUnitsPerGranule);
+  while (q < end) {
+    if (q / kUnitsPerGranule >= segs[seg + 1].granule_begin)
+      seg = search_segment(segs, seg + 1, nseg, q / kUnitsPerGranule);
+    const SegDesc d = segs[seg];
+    const uint64_t begin = d.granule_begin * kUnitsPerGranule;
+    // where the segment's whole vectors (FP8: pairs of units) end
+    uint64_t whole = begin + d.numel / Io::kVec * Io::kVec / kUnit;
+    if (whole > end) whole = end;
+    if (q + kTile <= whole && blockDim.x == kShape.threads) {
+      const uint64_t e = (q - begin) * kUnit, g = d.index_base + e;
+      // tiles before the high counter word changes (g passes a multiple of 2^34)
+      const uint64_t same_hi = ((((g >> 34) + 1) << 34) - g) / kUnit;
+      uint64_t tiles = (whole - q < same_hi ? whole - q : same_hi) / kTile;
+      if (tiles > 0) {
+        if (tiles > 0x7FFFFFFFu) tiles = 0x7FFFFFFFu;
+        const uint64_t mine = threadIdx.x * static_cast<uint64_t>(Io::kVec);
+        axpy_run<Io, kMode>(static_cast<typename Io::Scalar*>(d.data) + e + mine, (g + mine) >> 2,
+                            static_cast<uint32_t>(tiles), a, Io::kScaled ? inv_scale[seg] : 1.0f);
+        q += tiles * kTile;
+        continue;
+      }
+    }
+    const uint64_t stop = q + kTile < end ? q + kTile : end;
+    const int last = search_segment(segs, seg, nseg, (stop - 1) / kUnitsPerGranule);
+    axpy_units<Io, kMode>(segs, inv_scale, seg, last, q, stop, a);
+    __syncwarp();
+    q = stop;
+    seg = last;
   }
 }
 
 // Seeds of an update launch are staged in shared memory kSchedRows at a time,
 // one row of kRowVecs 16-byte words per seed, filled by the CTA for the
-// high counter word j_hi of the tile at hand:
+// high counter word j_hi of the units at hand:
 //   row[0] = (k0, k1, round 1's k0, tile constant x2)
-//   row[1] = (tile constant lo2, coefficient bits, 0, 0)
+//   row[1] = (tile constant lo2, coefficient bits, round 1's k1, 0)
 //   row[2 .. 5] = round keys of rounds 2..9
 // so a seed costs its thread six shared-memory loads instead of deriving its
 // key schedule and tile constants. Row kSchedRows is the trailing perturb's.
@@ -581,7 +566,7 @@ __device__ __forceinline__ void fill_row(SchedRow& row, uint32_t k0, uint32_t k1
   const PhiloxSched s = philox_sched(static_cast<uint64_t>(k1) << 32 | k0);
   const TileConst t = tile_const(j_hi, s.rk[0], s.rk[3]);
   row[0] = make_uint4(s.rk[0], s.rk[1], s.rk[2], t.x2);
-  row[1] = make_uint4(t.lo2, __float_as_uint(coeff), 0u, 0u);
+  row[1] = make_uint4(t.lo2, __float_as_uint(coeff), s.rk[3], 0u);
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     row[2 + k] = make_uint4(s.rk[4 + 4 * k], s.rk[5 + 4 * k], s.rk[6 + 4 * k], s.rk[7 + 4 * k]);
@@ -593,24 +578,21 @@ struct KeyRegs {
   __device__ uint32_t operator[](int i) const { return k[i]; }
 };
 
-// Generator and coefficient of one staged row.
+// Generator of one staged row. kUniformHi: the units at hand share the row's
+// high counter word; otherwise the thread's own one is j_hi.
 template <bool kUniformHi>
-__device__ __forceinline__ auto row_gen(const SchedRow& row) {
+__device__ __forceinline__ SchedGen<KeyRegs> row_gen(const SchedRow& row, uint32_t j_hi) {
   const uint4 r0 = row[0], r1 = row[1];
-  if constexpr (kUniformHi) {
-    KeyRegs kr;
+  KeyRegs kr;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint4 w = row[2 + k];
-      kr.k[4 * k] = w.x;
-      kr.k[4 * k + 1] = w.y;
-      kr.k[4 * k + 2] = w.z;
-      kr.k[4 * k + 3] = w.w;
-    }
-    return SchedGen<KeyRegs>{TileConst{r0.w, r1.x}, r0.y, r0.z, kr};
-  } else {
-    return AnyGen{PhiloxKey{r0.x, r0.y}};
+  for (int k = 0; k < 4; ++k) {
+    const uint4 w = row[2 + k];
+    kr.k[4 * k] = w.x;
+    kr.k[4 * k + 1] = w.y;
+    kr.k[4 * k + 2] = w.z;
+    kr.k[4 * k + 3] = w.w;
   }
+  return {kUniformHi ? TileConst{r0.w, r1.x} : tile_const(j_hi, r0.x, r1.z), r0.y, r0.z, kr};
 }
 
 __device__ __forceinline__ float row_coeff(const SchedRow& row) { return __uint_as_float(row[1].y); }
@@ -629,189 +611,184 @@ __device__ __forceinline__ void ensure_rows(SchedRow* s_rows, RowState& rs, cons
   if (rs.first == c0 && rs.j_hi == j_hi) return;
   __syncthreads();  // every thread is done with the rows held so far
   const int m = args.n - c0 < kSchedRows ? args.n - c0 : kSchedRows;
-  for (int k = threadIdx.x; k < m; k += kBlockThreads)
+  for (int k = threadIdx.x; k < m; k += blockDim.x)
     fill_row(s_rows[k], args.key[c0 + k][0], args.key[c0 + k][1], args.coeff[c0 + k], j_hi);
-  if (kPerturb && threadIdx.x == kBlockThreads - 1)
+  if (kPerturb && threadIdx.x == blockDim.x - 1)
     fill_row(s_rows[kSchedRows], args.pkey[0], args.pkey[1], args.pscale, j_hi);
   __syncthreads();
   rs.first = c0;
   rs.j_hi = j_hi;
 }
 
-// acc[q] += c_i eps_i over the seeds i of [c0, c1) held in the rows from c0,
-// for the thread's vectors u0 .. u0 + G - 1 (ascending i).
-template <class Io, bool kUniformHi, int G>
-__device__ __forceinline__ void accumulate_seeds(const TileRef<Io>& r, int u0, const SchedRow* rows,
-                                                 int count, float (&acc)[G][Io::kVec]) {
-  constexpr int V = Io::kVec;
-  constexpr int kUnroll = ES_SEED_UNROLL;
-  if constexpr (kUpdatePipelined && G == 1 && V <= 8) {
-    // Software-pipelined over the seeds: seed i + 1's Philox words are
-    // computed in the same basic block as seed i's transform, so the
-    // integer-multiply phase of one seed overlaps the MUFU/FP32 phase of the
-    // other.
-    constexpr int NB = V / 4;
-    const uint64_t e = vec_elem(r, u0);
-    if (e >= r.numel || count < 1) return;
-    const uint64_t j0 = (r.index_base + e) >> 2;
-    // round 0's products, shared by every seed (kRound0)
-    constexpr bool kR0 = kUniformHi && kRound0 >= 1;
-    Round0 p0[NB];
+// raw <- round(raw + acc) in storage form; acc <- 0.
+template <class Io>
+__device__ __forceinline__ void apply_acc(typename Io::Raw& raw, float (&acc)[kUnit], float inv) {
+  float f[kUnit];
+  Io::unpack_unit(raw, f);
 #pragma unroll
-    for (int b = 0; b < NB; ++b)
-      p0[b] = kR0 ? philox_round0<false>(static_cast<uint32_t>(j0 + b)) : Round0{0u, 0u};
-    auto words = [&](const SchedRow& row, uint4 (&w)[NB]) {
-      const auto gen = row_gen<kUniformHi>(row);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        if constexpr (kR0) w[b] = gen.block_r0(p0[b]);
-        else w[b] = gen.block(j0 + b);
-      }
-    };
-    auto transform = [&](const uint4 (&w)[NB], const SchedRow& row) {
-      add_scaled_noise_words<kUpdateForm, V>(w, row_coeff(row), acc[0]);
-    };
-    uint4 x[NB];
-    words(rows[0], x);
-    if constexpr (kUpdatePingPong) {
-      // two seeds per iteration, the word buffers alternating, so no copies
-      uint4 y[NB];
-      int i = 0;
-#pragma unroll 1
-      for (; i + 2 < count; i += 2) {
-        words(rows[i + 1], y);
-        transform(x, rows[i]);
-        words(rows[i + 2], x);
-        transform(y, rows[i + 1]);
-      }
-      if (i + 1 < count) {
-        words(rows[i + 1], y);
-        transform(x, rows[i]);
-        transform(y, rows[i + 1]);
-      } else {
-        transform(x, rows[i]);
-      }
-    } else {
-#pragma unroll 1
-      for (int i = 0; i + 1 < count; ++i) {
-        uint4 xn[NB];
-        words(rows[i + 1], xn);
-        transform(x, rows[i]);
-#pragma unroll
-        for (int b = 0; b < NB; ++b) x[b] = xn[b];
-      }
-      transform(x, rows[count - 1]);
-    }
-  } else {
-#pragma unroll kUnroll
-    for (int i = 0; i < count; ++i) {
-      const auto gen = row_gen<kUniformHi>(rows[i]);
-      const float c = row_coeff(rows[i]);
-#pragma unroll
-      for (int q = 0; q < G; ++q) {
-        const uint64_t e = vec_elem(r, u0 + q);
-        if (e >= r.numel) continue;
-        add_scaled_noise<kUpdateForm, V>(gen, (r.index_base + e) >> 2, c, acc[q]);
-      }
-    }
+  for (int k = 0; k < kUnit; ++k) {
+    f[k] = add_acc<Io>(f[k], acc[k], inv);
+    acc[k] = 0.0f;
   }
+  raw = Io::pack_unit(f);
 }
 
-// v[q] <- round(v[q] + acc[q]) in storage form; acc <- 0.
-template <class Io, int G>
-__device__ __forceinline__ void apply_acc(uint4 (&v)[G], float (&acc)[G][Io::kVec], float inv) {
-#pragma unroll
-  for (int q = 0; q < G; ++q) {
-    float f[Io::kVec];
-    Io::unpack(v[q], f);
-#pragma unroll
-    for (int k = 0; k < Io::kVec; ++k) {
-      f[k] = add_acc<Io>(f[k], acc[q][k], inv);
-      acc[q][k] = 0.0f;
-    }
-    v[q] = Io::pack(f);
-  }
-}
-
-// One tile of a fused update launch, G vectors at a time. Theta stays in
-// registers in storage form; generation g adds acc_g = sum_{i in g} c_i eps_i
-// (fp32, ascending i) and rounds once, exactly as a separate launch per
-// generation would store it (kSingle: one generation, and with kPerturb the
-// next generation's first perturb follows, rounded again). Theta is read and
-// written once.
-template <class Io, bool kUniformHi, bool kSingle, bool kPerturb, int G>
-__device__ __forceinline__ void update_tile(const TileRef<Io>& r, const UpdateArgs& args,
+// A thread's unit in a fused update launch. Theta stays in registers in
+// storage form; generation g adds acc_g = sum_{i in g} c_i eps_i (fp32,
+// ascending i) and rounds once, exactly as a separate launch per generation
+// would store it (kSingle: one generation, and with kPerturb the next
+// generation's first perturb follows, rounded again).
+// The loop over the seeds is software-pipelined: seed i + 1's Philox words are
+// computed in the same basic block as seed i's transform, so the integer
+// multiplies of one seed overlap the MUFU and FP32 work of the other, on
+// alternating word buffers (no copies).
+template <class Io, bool kUniformHi, bool kSingle, bool kPerturb>
+__device__ __forceinline__ void update_unit(typename Io::Scalar* p, int rem, float inv,
+                                            uint32_t my_hi, const Round0 (&p0)[kUnit / 4],
+                                            uint32_t j_hi, const UpdateArgs& args,
                                             SchedRow* s_rows, RowState& rs) {
-  constexpr int V = Io::kVec;
-  const uint32_t j_hi = static_cast<uint32_t>((r.index_base + r.t0) >> 34);
+  constexpr int NB = kUnit / 4;
   const int n = args.n;
-#pragma unroll 1
-  for (int u0 = 0; u0 < kVecsPerThread; u0 += G) {
-    uint4 v[G];
-    load_group<Io, G>(r, u0, v);
-    float acc[G][V];
+  typename Io::Raw raw = Io::zero_unit();
+  if (rem > 0) raw = Io::load_unit(p, rem);
+  float acc[kUnit];
 #pragma unroll
-    for (int q = 0; q < G; ++q)
+  for (int k = 0; k < kUnit; ++k) acc[k] = 0.0f;
+  auto words = [&](const SchedRow& row, uint4 (&w)[NB]) {
+    const auto gen = row_gen<kUniformHi>(row, my_hi);
 #pragma unroll
-      for (int k = 0; k < V; ++k) acc[q][k] = 0.0f;
-    int g = 0;
+    for (int b = 0; b < NB; ++b) w[b] = gen.block_r0(p0[b]);
+  };
+  int g = 0;
+  int gen_end = kSingle ? n : args.gen_end[0];
 #pragma unroll 1
-    for (int c0 = 0; c0 < n; c0 += kSchedRows) {
-      ensure_rows<kPerturb>(s_rows, rs, args, c0, j_hi);
-      const int c1 = n - c0 < kSchedRows ? n : c0 + kSchedRows;
-      if constexpr (kSingle) {
-        accumulate_seeds<Io, kUniformHi, G>(r, u0, s_rows, c1 - c0, acc);
-      } else {
-        // generation by generation within the chunk (generations are never empty)
-        int i = c0;
-        while (i < c1) {
-          const int end = args.gen_end[g] < c1 ? args.gen_end[g] : c1;
-          accumulate_seeds<Io, kUniformHi, G>(r, u0, s_rows + (i - c0), end - i, acc);
-          i = end;
-          if (i == args.gen_end[g]) {
-            apply_acc<Io, G>(v, acc, r.inv);
-            ++g;
-          }
+  for (int c0 = 0; c0 < n; c0 += kSchedRows) {
+    ensure_rows<kPerturb>(s_rows, rs, args, c0, j_hi);
+    const int count = n - c0 < kSchedRows ? n - c0 : kSchedRows;
+    if (rem <= 0) continue;
+    // seed i of the chunk; at a generation's last seed theta takes the sum
+    auto transform = [&](const uint4 (&w)[NB], int i) {
+      add_scaled_noise<kUnit>(w, row_coeff(s_rows[i]), acc);
+      if constexpr (!kSingle) {
+        if (c0 + i + 1 == gen_end) {
+          apply_acc<Io>(raw, acc, inv);
+          if (++g < args.n_gen) gen_end = args.gen_end[g];
         }
       }
+    };
+    uint4 x[NB], y[NB];
+    words(s_rows[0], x);
+    int i = 0;
+#pragma unroll 1
+    for (; i + 2 < count; i += 2) {
+      words(s_rows[i + 1], y);
+      transform(x, i);
+      words(s_rows[i + 2], x);
+      transform(y, i + 1);
     }
-    if constexpr (kSingle) apply_acc<Io, G>(v, acc, r.inv);
-    if constexpr (kPerturb) {
-      const auto pgen = row_gen<kUniformHi>(s_rows[kSchedRows]);
-      const float ps = row_coeff(s_rows[kSchedRows]) * r.inv;
-#pragma unroll
-      for (int q = 0; q < G; ++q) {
-        const uint64_t e = vec_elem(r, u0 + q);
-        if (e >= r.numel) continue;
-        float f[V];
-        Io::unpack(v[q], f);
-        add_scaled_noise<kUpdateForm, V>(pgen, (r.index_base + e) >> 2, ps, f);
-        v[q] = Io::pack(f);
-      }
+    if (i + 1 < count) {
+      words(s_rows[i + 1], y);
+      transform(x, i);
+      transform(y, i + 1);
+    } else {
+      transform(x, i);
     }
-#pragma unroll
-    for (int q = 0; q < G; ++q) store_vec(r, vec_elem(r, u0 + q), v[q]);
   }
+  if (rem <= 0) return;
+  if constexpr (kSingle) apply_acc<Io>(raw, acc, inv);
+  if constexpr (kPerturb) {
+    float f[kUnit];
+    Io::unpack_unit(raw, f);
+    uint4 x[NB];
+    words(s_rows[kSchedRows], x);
+    add_scaled_noise<kUnit>(x, row_coeff(s_rows[kSchedRows]) * inv, f);
+    raw = Io::pack_unit(f);
+  }
+  Io::store_unit(p, rem, raw);
 }
 
 // Fused update launch (es_update, es_replay, es_update_perturb): for each
 // generation g, theta[g] <- round(theta[g] + sum_{i in g} c_i eps_{s_i}[g]),
 // then with kPerturb theta <- round(theta + pscale * eps_pseed).
 // kSingle: one generation; otherwise args.n_gen generations, never empty.
+// A CTA walks its range a row at a time, one unit per thread (8 elements, two
+// independent Philox chains, in every storage type): runs of whole rows inside
+// one segment from a pointer and a counter that are stepped, and
+// single rows, each thread finding its own segment, where a segment, the range
+// or a high counter word ends.
+// Bound by the generator like the passes above. Measured over 792,680,960
+// parameters (ms; 3 CTAs of 256 threads on grid-stride tiles -> one CTA of 640):
+// 8 seeds bf16 4.70 -> 4.43 (1.43e12 Gaussians/s), fp32 5.32 -> 4.42 and FP8
+// 4.90 -> 4.41 (their seed loops were not pipelined: they took 8 elements in another form), 16 seeds +
+// perturb bf16 9.77 -> 9.20, 2 seeds bf16 1.48 -> 1.30. Several generations run fastest
+// with 768: 8 generations of 2 seeds 10.59 -> 9.41.
+template <bool kSingle>
+__host__ __device__ constexpr int update_threads() {
+  return kSingle ? 640 : 768;
+}
+
 template <class Io, bool kSingle, bool kPerturb>
-__global__ void __launch_bounds__(kBlockThreads, update_min_blocks())
-update_kernel(const SegDesc* __restrict__ segs, const float* __restrict__ inv_scale,
-              uint64_t total_tiles, const __grid_constant__ UpdateArgs args) {
-  constexpr int G = group_for<Io>(kUpdateGroup);
+__global__ void __launch_bounds__(update_threads<kSingle>(), 1)
+update_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
+              const Split split, const __grid_constant__ UpdateArgs args) {
+  constexpr int NB = kUnit / 4;
   __shared__ SchedRow s_rows[kSchedRows + 1];
   RowState rs{-1, 0u};
-  int seg = 0;
-  for (uint64_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-    const TileRef<Io> r = tile_ref<Io>(segs, inv_scale, seg, tile);
-    if (uniform_hi(r.index_base, r.t0, static_cast<uint64_t>(kBlockThreads) * kVecsPerThread * Io::kVec, r.numel))
-      update_tile<Io, true, kSingle, kPerturb, G>(r, args, s_rows, rs);
+  const uint32_t row = blockDim.x;
+  uint64_t q = range_begin(split) * kUnitsPerGranule;
+  const uint64_t end = range_end(split) * kUnitsPerGranule;
+  int seg = search_segment(segs, 0, nseg, q / kUnitsPerGranule);
+#pragma unroll 1
+  while (q < end) {
+    if (q / kUnitsPerGranule >= segs[seg + 1].granule_begin)
+      seg = search_segment(segs, seg + 1, nseg, q / kUnitsPerGranule);
+    const SegDesc d = segs[seg];
+    const uint64_t begin = d.granule_begin * kUnitsPerGranule;
+    uint64_t whole = begin + d.numel / kUnit;  // where the segment's whole units end
+    if (whole > end) whole = end;
+    const uint64_t e = (q - begin) * kUnit, index = d.index_base + e;
+    const uint32_t j_hi = static_cast<uint32_t>(index >> 34);
+    if (q + row <= whole) {
+      // rows before the high counter word changes (index passes a multiple of 2^34)
+      const uint64_t same_hi = ((((index >> 34) + 1) << 34) - index) / kUnit;
+      uint64_t rows = (whole - q < same_hi ? whole - q : same_hi) / row;
+      if (rows > 0) {
+        q += rows * row;
+        typename Io::Scalar* p =
+            static_cast<typename Io::Scalar*>(d.data) + e + threadIdx.x * kUnit;
+        const float inv = Io::kScaled ? inv_scale[seg] : 1.0f;
+        const uint32_t j0 = static_cast<uint32_t>(index >> 2) + threadIdx.x * NB;
+        Round0 p0[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) p0[b] = philox_round0<false>(j0 + b);
+#pragma unroll 1
+        for (;;) {
+          update_unit<Io, true, kSingle, kPerturb>(p, kUnit, inv, j_hi, p0, j_hi, args, s_rows, rs);
+          if (--rows == 0) break;
+          p += row * kUnit;
+#pragma unroll
+          for (int b = 0; b < NB; ++b) p0[b] = round0_step(p0[b], row * NB);
+        }
+        continue;
+      }
+    }
+    const uint64_t stop = q + row < end ? q + row : end;
+    const int last = search_segment(segs, seg, nseg, (stop - 1) / kUnitsPerGranule);
+    const uint64_t mine = q + threadIdx.x < stop ? q + threadIdx.x : stop - 1;
+    const UnitRef<Io> r = unit_ref<Io>(
+        segs, inv_scale, segment_between(segs, seg, last, mine / kUnitsPerGranule), mine);
+    const int rem = q + threadIdx.x < stop ? r.rem : 0;
+    Round0 p0[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) p0[b] = philox_round0<false>(static_cast<uint32_t>(r.j0 + b));
+    const uint32_t my_hi = static_cast<uint32_t>(r.j0 >> 32);
+    // the staged constants are those of the row's first unit
+    if (__syncthreads_and(rem == 0 || my_hi == j_hi))
+      update_unit<Io, true, kSingle, kPerturb>(r.p, rem, r.inv, my_hi, p0, j_hi, args, s_rows, rs);
     else
-      update_tile<Io, false, kSingle, kPerturb, G>(r, args, s_rows, rs);
+      update_unit<Io, false, kSingle, kPerturb>(r.p, rem, r.inv, my_hi, p0, j_hi, args, s_rows, rs);
+    q = stop;
+    seg = last;
   }
 }
 
@@ -842,17 +819,23 @@ noise_fill_kernel(uint64_t index_base, uint64_t n, PhiloxKey key, float* __restr
 // launch's schedule, the Philox constants of the blocks' high word per tile
 // (when the tile stays within one 2^32-block range), the packed transform with
 // the near-one series on a rare branch (values equal to box_muller's).
+constexpr int kFillBlocks = 4;  // Philox blocks per thread and tile
+
 template <bool kUniformHi>
 __device__ __forceinline__ void noise_fill_tile(uint64_t j_first, uint64_t b0, uint64_t nblocks,
                                                 const PhiloxSched& sched,
                                                 float4* __restrict__ out) {
-  const auto gen = sched_gen<kUniformHi>(sched, static_cast<uint32_t>((j_first + b0) >> 32));
+  const uint32_t j_hi = static_cast<uint32_t>((j_first + b0) >> 32);
 #pragma unroll
-  for (int q = 0; q < kVecsPerThread; ++q) {
+  for (int q = 0; q < kFillBlocks; ++q) {
     const uint64_t b = b0 + static_cast<uint64_t>(q * kBlockThreads + threadIdx.x);
     if (b < nblocks) {
+      const uint64_t j = j_first + b;
+      const auto gen =
+          sched_gen<false>(sched, kUniformHi ? j_hi : static_cast<uint32_t>(j >> 32));
+      const uint4 x[1] = {gen.block_r0(philox_round0<false>(static_cast<uint32_t>(j)))};
       Polar2 pp[1];
-      polar_blocks<NoiseForm::kPacked, 1>(gen, j_first + b, pp);
+      polar_from_words<1>(x, pp);
       const Polar2& p = pp[0];
       const float2 lo = __fmul2_rn(make_float2(-p.r.x, -p.r.x), make_float2(p.c.x, p.s.x));
       const float2 hi = __fmul2_rn(make_float2(-p.r.y, -p.r.y), make_float2(p.c.y, p.s.y));
@@ -864,7 +847,7 @@ __device__ __forceinline__ void noise_fill_tile(uint64_t j_first, uint64_t b0, u
 __global__ void __launch_bounds__(kBlockThreads)
 noise_fill_vec_kernel(uint64_t j_first, uint64_t nblocks, const __grid_constant__ PhiloxSched sched,
                       float4* __restrict__ out) {
-  constexpr uint64_t kTileBlocks = static_cast<uint64_t>(kBlockThreads) * kVecsPerThread;
+  constexpr uint64_t kTileBlocks = static_cast<uint64_t>(kBlockThreads) * kFillBlocks;
   const uint64_t tiles = (nblocks + kTileBlocks - 1) / kTileBlocks;
   for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const uint64_t b0 = tile * kTileBlocks;
@@ -932,7 +915,7 @@ std::mutex g_grid_mutex;
 GridEntry g_grid_cache[kGridCacheSize];
 int g_grid_used = 0;
 
-int resident_ctas(const void* kernel, int dev) {
+int resident_ctas(const void* kernel, int threads, int dev) {
   {
     std::lock_guard<std::mutex> lock(g_grid_mutex);
     for (int k = 0; k < g_grid_used; ++k)
@@ -941,7 +924,7 @@ int resident_ctas(const void* kernel, int dev) {
   }
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlockThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
   if (sms < 1) sms = 1;
   if (per_sm < 1) per_sm = 1;
   const int ctas = sms * per_sm;
@@ -956,20 +939,55 @@ template <class K>
 int persistent_grid(K kernel, uint64_t work_items) {
   int dev = 0;
   cudaGetDevice(&dev);
-  uint64_t grid = static_cast<uint64_t>(resident_ctas(reinterpret_cast<const void*>(kernel), dev));
+  uint64_t grid = static_cast<uint64_t>(resident_ctas(reinterpret_cast<const void*>(kernel), kBlockThreads, dev));
   if (work_items < grid) grid = work_items;
   return grid < 1 ? 1 : static_cast<int>(grid);
 }
 
-template <class Io, bool kTwo, bool kSame>
+// A streaming launch: its division, grid and block size.
+struct Launch {
+  Split split;
+  int grid, block;
+};
+
+// One range per resident CTA, in whole 8-granule pieces (256 bytes of bf16) so
+// that ranges meet at cache-line boundaries, and no less than a warp's units.
+// Where the ranges are shorter than `whole_block` units the block shrinks to
+// what they need, in rows of equal length (a multiple of 128 threads above
+// 128: each SM sub-partition then holds as many warps as the others; 448 and
+// 576 threads measured 10 % slower than 384 and 512).
+Launch make_launch(const void* kernel, int threads, uint64_t whole_block, uint64_t granules) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const uint64_t ctas = static_cast<uint64_t>(resident_ctas(kernel, threads, dev));
+  uint64_t per = (granules + ctas - 1) / ctas;
+  per = (per + 7) / 8 * 8;
+  if (per < 32 / kUnitsPerGranule) per = 32 / kUnitsPerGranule;
+  Launch l;
+  l.split = Split{granules, per};
+  l.grid = static_cast<int>((granules + per - 1) / per);
+  l.block = threads;
+  const uint64_t units = per * kUnitsPerGranule;
+  if (units < whole_block) {
+    const uint64_t rows = (units + threads - 1) / threads;
+    const uint64_t want = (units + rows - 1) / rows;
+    const uint64_t step = want > 128 ? 128 : 32;
+    const uint64_t block = (want + step - 1) / step * step;
+    l.block = static_cast<int>(block < static_cast<uint64_t>(threads) ? block : threads);
+  }
+  return l;
+}
+
+template <class Io, AxpyMode kMode>
 cudaError_t launch_axpy_io(const PlanView& plan, const AxpyArgs& a, cudaStream_t stream) {
-  auto k = axpy_noise_kernel<Io, kTwo, kSame>;
-  k<<<persistent_grid(k, plan.total_tiles), kBlockThreads, 0, stream>>>(
-      plan.segs, plan.inv_scale, plan.total_tiles, a);
+  auto k = axpy_noise_kernel<Io, kMode>;
+  const Launch l = make_launch(reinterpret_cast<const void*>(k), axpy_shape<Io, kMode>().threads,
+                               axpy_tile_units<Io, kMode>(), plan.granules);
+  k<<<l.grid, l.block, 0, stream>>>(plan.segs, plan.nseg, plan.inv_scale, l.split, a);
   return cudaGetLastError();
 }
 
-template <bool kTwo, bool kSame>
+template <AxpyMode kMode>
 cudaError_t launch_axpy(const PlanView& plan, uint64_t seed, float scale, uint64_t seed2,
                         float scale2, cudaStream_t stream) {
   AxpyArgs a;
@@ -977,37 +995,45 @@ cudaError_t launch_axpy(const PlanView& plan, uint64_t seed, float scale, uint64
   a.s2 = philox_sched(seed2);
   a.scale1 = scale;
   a.scale2 = scale2;
-  if (plan.dtype == ES_BF16) return launch_axpy_io<Bf16Io, kTwo, kSame>(plan, a, stream);
-  if (plan.dtype == ES_FP8_E4M3) return launch_axpy_io<Fp8Io, kTwo, kSame>(plan, a, stream);
-  return launch_axpy_io<F32Io, kTwo, kSame>(plan, a, stream);
+  if (plan.dtype == ES_BF16) return launch_axpy_io<Bf16Io, kMode>(plan, a, stream);
+  if (plan.dtype == ES_FP8_E4M3) return launch_axpy_io<Fp8Io, kMode>(plan, a, stream);
+  return launch_axpy_io<F32Io, kMode>(plan, a, stream);
 }
 
 }  // namespace
 
 cudaError_t launch_axpy_noise(const PlanView& plan, uint64_t seed, float scale,
                               cudaStream_t stream) {
-  return launch_axpy<false, false>(plan, seed, scale, 0u, 0.0f, stream);
+  return launch_axpy<AxpyMode::kOne>(plan, seed, scale, 0u, 0.0f, stream);
 }
 
 cudaError_t launch_axpy_noise2(const PlanView& plan, uint64_t seed, float scale, uint64_t seed2,
                                float scale2, cudaStream_t stream) {
-  if (seed == seed2) return launch_axpy<true, true>(plan, seed, scale, seed2, scale2, stream);
-  return launch_axpy<true, false>(plan, seed, scale, seed2, scale2, stream);
+  if (seed == seed2)
+    return launch_axpy<AxpyMode::kFlip>(plan, seed, scale, seed2, scale2, stream);
+  return launch_axpy<AxpyMode::kTwo>(plan, seed, scale, seed2, scale2, stream);
 }
 
-template <class Io>
+template <class Io, bool kSingle, bool kPerturb>
 cudaError_t launch_update_io(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
-  auto k = update_kernel<Io, false, false>;
-  if (args.n_gen == 1) k = args.perturb ? update_kernel<Io, true, true> : update_kernel<Io, true, false>;
-  k<<<persistent_grid(k, plan.total_tiles), kBlockThreads, 0, stream>>>(
-      plan.segs, plan.inv_scale, plan.total_tiles, args);
+  auto k = update_kernel<Io, kSingle, kPerturb>;
+  constexpr int kThreads = update_threads<kSingle>();
+  const Launch l = make_launch(reinterpret_cast<const void*>(k), kThreads, 4 * kThreads, plan.granules);
+  k<<<l.grid, l.block, 0, stream>>>(plan.segs, plan.nseg, plan.inv_scale, l.split, args);
   return cudaGetLastError();
 }
 
+template <class Io>
+cudaError_t launch_update_dtype(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
+  if (args.n_gen > 1) return launch_update_io<Io, false, false>(plan, args, stream);
+  return args.perturb ? launch_update_io<Io, true, true>(plan, args, stream)
+                      : launch_update_io<Io, true, false>(plan, args, stream);
+}
+
 cudaError_t launch_update(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
-  if (plan.dtype == ES_BF16) return launch_update_io<Bf16Io>(plan, args, stream);
-  if (plan.dtype == ES_FP8_E4M3) return launch_update_io<Fp8Io>(plan, args, stream);
-  return launch_update_io<F32Io>(plan, args, stream);
+  if (plan.dtype == ES_BF16) return launch_update_dtype<Bf16Io>(plan, args, stream);
+  if (plan.dtype == ES_FP8_E4M3) return launch_update_dtype<Fp8Io>(plan, args, stream);
+  return launch_update_dtype<F32Io>(plan, args, stream);
 }
 
 cudaError_t launch_noise_bits(uint64_t seed, uint64_t block_base, uint64_t nblocks,
@@ -1035,7 +1061,7 @@ cudaError_t launch_noise_fill(uint64_t seed, uint64_t index_base, uint64_t n, fl
   // left over go through the general kernel below.
   if (reinterpret_cast<uintptr_t>(out) % 16 == 0 && index_base % 4 == 0 && n >= 4) {
     const uint64_t full = n / 4;
-    constexpr uint64_t kTileBlocks = static_cast<uint64_t>(kBlockThreads) * kVecsPerThread;
+    constexpr uint64_t kTileBlocks = static_cast<uint64_t>(kBlockThreads) * kFillBlocks;
     const int grid = persistent_grid(noise_fill_vec_kernel, (full + kTileBlocks - 1) / kTileBlocks);
     noise_fill_vec_kernel<<<grid, kBlockThreads, 0, stream>>>(index_base / 4, full,
                                                               philox_sched(seed),

@@ -143,13 +143,12 @@ extern "C" es_status_t es_perturb_noalloc(const es_segment_t* segs, int nseg, es
                     order[k], order[k + 1]);
 
   SegDesc table[ES_STATIC_MAX_SEGMENTS + 1];
-  const uint64_t tile = esopt::tile_elems(dtype);
-  uint64_t tiles = 0;
+  uint64_t granules = 0;
   for (int k = 0; k < nseg; ++k) {
-    table[k] = SegDesc{segs[k].data, segs[k].numel, segs[k].index_base, tiles};
-    tiles += (segs[k].numel + tile - 1) / tile;
+    table[k] = SegDesc{segs[k].data, segs[k].numel, segs[k].index_base, granules};
+    granules += esopt::granules_of(segs[k].numel);
   }
-  table[nseg] = SegDesc{nullptr, 0, 0, tiles};
+  table[nseg] = SegDesc{nullptr, 0, 0, granules};
 
   // The table is copied from this call's stack; a copy recorded into a graph
   // would read that memory again at every replay, long after it is gone. So a
@@ -187,7 +186,7 @@ extern "C" es_status_t es_perturb_noalloc(const es_segment_t* segs, int nseg, es
   err = cudaMemcpyAsync(d_table, table, (static_cast<size_t>(nseg) + 1) * sizeof(SegDesc),
                         cudaMemcpyHostToDevice, s);
   if (err != cudaSuccess) return reject(ES_ERR_CUDA, "es_perturb_noalloc: copy of the segment table failed");
-  err = esopt::launch_axpy_noise(esopt::PlanView{d_table, tiles, dtype, nullptr}, seed, sigma, s);
+  err = esopt::launch_axpy_noise(esopt::PlanView{d_table, nseg, granules, dtype, nullptr}, seed, sigma, s);
   if (err != cudaSuccess) return reject(ES_ERR_CUDA, "es_perturb_noalloc: kernel launch failed");
   return esopt::record_status(ES_OK, "");
 }

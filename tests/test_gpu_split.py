@@ -1,0 +1,96 @@
+"""How a launch's work is cut up: the segment search and the tile sizes at the
+sizes where they can go wrong, element by element against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from parity import noise_abs_tol
+from test_gpu_step import build_plan, compare, host_values, indices, make_params
+
+pytestmark = pytest.mark.gpu
+
+
+# The warp searches 32 table entries at a time: one step, the edges of one and two
+# steps, and three steps, with tiles of one segment, of many and of the last one.
+@pytest.mark.parametrize("nseg", [1, 2, 32, 33, 34, 65, 1023, 1026, 2500])
+def test_segment_search(es, oracle, nseg):
+    rng = np.random.default_rng(nseg)
+    numels = [int(n) for n in rng.integers(1, 70, size=nseg)]
+    numels[nseg // 2] = 3 * 8192 + 5
+    numels[-1] = 8193
+    tensors = make_params("bf16", numels, seed=nseg)
+    plan, segs = build_plan(es, tensors)
+    before = np.concatenate([host_values(t) for t in tensors])
+    g = np.concatenate(indices(segs))
+    es.es_perturb(plan, 21, 1e-3)
+    torch.cuda.synchronize()
+    got = np.concatenate([host_values(t) for t in tensors])
+    compare("bf16", got, oracle.perturb(before, g, 21, 1e-3, "bf16"), f"{nseg} segments",
+            noise_abs_tol([oracle.noise_at(21, g)], [1e-3]))
+    plan.close()
+
+
+# One segment long enough for runs of whole tiles and rows in every CTA, the
+# high counter word changing inside it, against the same memory as many short
+# segments (units found one by one): bit-identical everywhere, and equal to the
+# oracle around the change, at both ends and on a sample.
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "fp8"])
+@pytest.mark.parametrize("numel", [152 * 1024 * 64, 152 * 1024 * 64 + 4 * 1024 * 8 + 3])
+def test_long_runs_equal_short_segments(es, oracle, dtype, numel):
+    base = 2**34 - 8 * (numel // 17)
+    scale = 2.0**-9
+    if dtype == "fp8":
+        rng = np.random.default_rng(3)
+        codes = rng.integers(0, 120, size=numel).astype(np.uint8)
+        a = torch.from_numpy(codes).cuda()
+    else:
+        (a,) = make_params(dtype, [numel], seed=3)
+    b = a.clone()
+    step = 8 * 1111 if dtype != "fp8" else 16 * 555
+    pieces = [b[o:o + step] for o in range(0, numel, step)]
+    scales = [scale] if dtype == "fp8" else None
+    long_plan = es.plan_from_tensors([a], [base], scales)
+    short_plan = es.plan_from_tensors(pieces, [base + o for o in range(0, numel, step)],
+                                      scales and scales * len(pieces))
+    edge = 2**34 - base
+    at = np.unique(np.concatenate([
+        np.arange(64), np.arange(edge - 9000, edge + 9000), np.arange(numel - 9000, numel),
+        np.random.default_rng(4).integers(0, numel, size=20000)]))
+    g = np.uint64(base) + at.astype(np.uint64)
+    seeds = np.array([9, 2**40 + 1, 77], dtype=np.uint64)
+    coeffs = np.array([2e-3, -1e-3, 5e-4], dtype=np.float32)
+
+    def sample():
+        return a.cpu().numpy()[at] if dtype == "fp8" else host_values(a)[at]
+
+    def check(what, want, noise):
+        torch.cuda.synchronize()
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), what
+        if dtype == "fp8":
+            from test_gpu_fp8 import assert_e4m3_close
+            assert_e4m3_close(sample(), want, what, noise / scale)
+        else:
+            compare(dtype, sample(), want, what, noise)
+
+    def both(call):
+        before = sample()
+        call(long_plan)
+        call(short_plan)
+        return before
+
+    name, extra = ("e4m3", (scale,)) if dtype == "fp8" else (dtype, ())
+    tol = noise_abs_tol([oracle.noise_at(int(s), g) for s in seeds], [1e-3] * 3)
+    before = both(lambda p: es.es_perturb(p, 9, 1e-3))
+    check("perturb", oracle.perturb(before, g, 9, 1e-3, name, *extra), tol)
+    for second in (77, 9):
+        both(lambda p: es.es_restore_perturb(p, 9, 1e-3, second, -1e-3))
+        torch.cuda.synchronize()
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), "restore_perturb"
+    before = both(lambda p: es.es_update(p, seeds, coeffs))
+    check("update", oracle.update(before, g, seeds, coeffs, name, *extra), 2 * tol)
+    both(lambda p: es.es_update_perturb(p, seeds, coeffs, 5, 1e-3))
+    both(lambda p: es.es_replay(p, np.tile(seeds, 50), np.tile(coeffs, 50), [1, 2, 3] * 25))
+    torch.cuda.synchronize()
+    assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), "update_perturb, replay"
+    long_plan.close()
+    short_plan.close()
