@@ -19,7 +19,7 @@ constexpr uint64_t granules_of(uint64_t numel) {
   return numel / kGranule + (numel % kGranule != 0 ? 1u : 0u);
 }
 
-// Threads per CTA of the noise-fill and diagnostic kernels.
+// Threads per CTA of the diagnostic kernels (es_noise_bits, es_box_muller).
 constexpr int kBlockThreads = 256;
 
 // Bytes per element, per dtype.

@@ -395,13 +395,4 @@ __device__ __forceinline__ float2 box_muller(uint32_t xa, uint32_t xb) {
   return make_float2(-p.r * p.c, -p.r * p.s);
 }
 
-// eps[4j .. 4j+3] for one seed, materialised.
-__device__ __forceinline__ float4 gaussian4(uint64_t j, PhiloxKey key) {
-  const uint4 x = philox_block_tile(static_cast<uint32_t>(j),
-                                    philox_tile(static_cast<uint32_t>(j >> 32), key));
-  const float2 p = box_muller(x.x, x.y);
-  const float2 q = box_muller(x.z, x.w);
-  return make_float4(p.x, p.y, q.x, q.y);
-}
-
 }  // namespace esopt

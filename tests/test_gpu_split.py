@@ -94,3 +94,28 @@ def test_long_runs_equal_short_segments(es, oracle, dtype, numel):
     assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), "update_perturb, replay"
     long_plan.close()
     short_plan.close()
+
+
+# es_noise_fill for every way that index_base and out's 16-byte alignment can
+# meet: the smallest counts, the edges of a row of 32 groups and of a pair of
+# rows, and counts that fill every warp, across the change of the high counter
+# word; bit-identical to one aligned fill, which the oracle checks.
+@pytest.mark.parametrize("lead", [0, 1, 2, 3])
+def test_noise_fill_alignments(es, oracle, lead):
+    start = 2**34 - 4_000
+    whole = torch.empty(3_000_016, device="cuda")
+    es.es_noise_fill(31, start, whole.numel(), whole)
+    at = np.unique(np.concatenate([np.arange(8_000), np.arange(0, whole.numel(), 97)]))
+    want = oracle.noise_at(31, np.uint64(start) + at.astype(np.uint64))
+    got = whole.cpu().numpy()[at].astype(np.float64)
+    assert np.all(np.abs(got - want) <= 1e-5 * np.maximum(1.0, np.abs(want)))
+    out = torch.empty(3_000_032, device="cuda")
+    for skip in (0, 1, 2, 3, 3_998):
+        for n in (1, 2, 3, 4, 5, 127, 128, 129, 255, 256, 257, 4_001, 622_593, 3_000_001):
+            if skip + n > whole.numel():
+                continue
+            out.fill_(7.0)
+            es.es_noise_fill(31, start + skip, n, out[4 + lead:])
+            torch.cuda.synchronize()
+            assert torch.equal(out[4 + lead:4 + lead + n], whole[skip:skip + n]), (skip, n)
+            assert torch.all(out[:4 + lead] == 7.0) and torch.all(out[4 + lead + n:] == 7.0)
