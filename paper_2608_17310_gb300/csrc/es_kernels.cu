@@ -356,39 +356,78 @@ __device__ __forceinline__ UnitRef<Io> unit_ref(const SegDesc* __restrict__ segs
 
 // What a pass over the parameters does: one step theta += scale1 * eps_seed1;
 // two steps, the second on the first's result rounded to the storage type
-// (restore of one member fused with the perturb of the next); or the two steps
-// of one seed, whose noise is generated once (the antithetic flip).
-enum class AxpyMode { kOne, kTwo, kFlip };
+// (restore of one member fused with the perturb of the next); the two steps
+// of one seed, whose noise is generated once (the antithetic flip); or the update
+// of a population of 1 to 4, theta += sum_i scale_i eps_seed_i rounded once.
+enum class AxpyMode { kOne, kTwo, kFlip, kSum1, kSum2, kSum3, kSum4 };
+constexpr int kMaxSum = 4;
 
-// Arguments of a perturb/restore launch: the schedule and scale of each step
-// (step 2 unused by kOne). A __grid_constant__ parameter, so every round key
-// is read from the constant bank as an instruction operand.
+// Number of seeds of a mode, and whether it is one of the sums.
+__host__ __device__ constexpr int axpy_seeds(AxpyMode m) {
+  return m == AxpyMode::kOne || m == AxpyMode::kFlip || m == AxpyMode::kSum1 ? 1
+         : m == AxpyMode::kTwo || m == AxpyMode::kSum2                     ? 2
+         : m == AxpyMode::kSum3                                            ? 3
+                                                                           : 4;
+}
+__host__ __device__ constexpr bool axpy_is_sum(AxpyMode m) { return m >= AxpyMode::kSum1; }
+
+// Arguments of a launch: each seed's schedule, and the scale of each step or
+// seed. A __grid_constant__ parameter, so every round key is read from the
+// constant bank as an instruction operand.
 struct AxpyArgs {
-  PhiloxSched s1, s2;
-  float scale1, scale2;
+  PhiloxSched seed[kMaxSum];
+  float scale[kMaxSum];
 };
 
-// The steps of kMode on the V values f. words(second, x) gives the Philox words
-// of the first or the second seed's blocks.
+// The steps of kMode on the V values f. words(i, x) gives the Philox words of
+// seed i's blocks; inv is 1 / the segment's scale.
 template <class Io, AxpyMode kMode, int V, class Words>
-__device__ __forceinline__ void axpy_values(const Words& words, float s1, float s2, float (&f)[V]) {
+__device__ __forceinline__ void axpy_values(const Words& words, const AxpyArgs& a, float inv,
+                                            float (&f)[V]) {
   uint4 x[V / 4];
-  words(false, x);
-  if constexpr (kMode == AxpyMode::kFlip) {
+  if constexpr (axpy_is_sum(kMode)) {
+    float acc[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) acc[k] = 0.0f;
+#pragma unroll
+    for (int i = 0; i < axpy_seeds(kMode); ++i) {
+      words(i, x);
+      add_scaled_noise<V>(x, a.scale[i], acc);
+    }
+#pragma unroll
+    for (int k = 0; k < V; ++k) f[k] = add_acc<Io>(f[k], acc[k], inv);
+  } else if constexpr (kMode == AxpyMode::kFlip) {
+    words(0, x);
     Polar2 pp[V / 4];
     polar_from_words<V / 4>(x, pp);
-    apply_noise<V>(pp, s1, f);
+    apply_noise<V>(pp, a.scale[0] * inv, f);
     Io::round_trip(f);
-    apply_noise<V>(pp, s2, f);
+    apply_noise<V>(pp, a.scale[1] * inv, f);
   } else {
-    add_scaled_noise<V>(x, s1, f);
+    words(0, x);
+    add_scaled_noise<V>(x, a.scale[0] * inv, f);
     if constexpr (kMode == AxpyMode::kTwo) {
       Io::round_trip(f);
-      words(true, x);
-      add_scaled_noise<V>(x, s2, f);
+      words(1, x);
+      add_scaled_noise<V>(x, a.scale[1] * inv, f);
     }
   }
 }
+
+// The generators of a launch's seeds for one high counter word.
+template <AxpyMode kMode, bool kWide>
+struct AxpyGens {
+  static constexpr int kSeeds = axpy_seeds(kMode);
+  TileConst t[kSeeds];
+  __device__ AxpyGens(const AxpyArgs& a, uint32_t j_hi) {
+#pragma unroll
+    for (int i = 0; i < kSeeds; ++i) t[i] = tile_const(j_hi, a.seed[i].rk[0], a.seed[i].rk[3]);
+  }
+  __device__ uint4 words(const AxpyArgs& a, int i, Round0 p0) const {
+    const uint32_t* rk = a.seed[i].rk;
+    return philox_block_r0<kWide>(p0, t[i], rk[1], rk[2], rk + 4);
+  }
+};
 
 // Shape of a pass: threads of its one CTA per SM, 16-byte vectors per thread
 // in a tile (the unrolled body of the loop) and how many vectors ahead theta is
@@ -400,6 +439,10 @@ __device__ __forceinline__ void axpy_values(const Words& words, float s1, float 
 // vectors, 1 ahead, grid-stride tiles -> this): bf16 one step 678 -> 569 (5.58 TB/s), two
 // steps 1217 -> 1094 (1.449e12 Gaussians/s), flip 729 -> 621; fp32 971 -> 962 (6.59 TB/s: HBM),
 // 1366 -> 1077, 976 -> 961; FP8 636 -> 575, 1301 -> 1127, 718 -> 639.
+// The sums replace the seed loop of update_kernel where it is too short for its
+// pipeline: 1 / 2 / 3 / 4 seeds bf16 972 / 1480 / 2035 / 2555 -> 591 / 1094 /
+// 1599 / 2143, fp32 1125 / 1642 / 2253 / 2866 -> 962 / 1088 / 1589 / 2145, FP8
+// 811 / 1392 / 1979 / 2567 -> 602 / 1110 / 1608 / 2113.
 // Thread counts that are no multiple of 128 leave the SM's four schedulers
 // unequal warps and run 10 % slower.
 struct AxpyShape {
@@ -407,6 +450,11 @@ struct AxpyShape {
 };
 template <class Io, AxpyMode kMode>
 __host__ __device__ constexpr AxpyShape axpy_shape() {
+  if (axpy_is_sum(kMode)) {
+    if (Io::kVec == 4) return {1024, 4, 2};
+    if (Io::kVec == 16) return {kMode == AxpyMode::kSum1 ? 768 : 512, 1, 1};
+    return kMode == AxpyMode::kSum4 ? AxpyShape{768, 1, 1} : AxpyShape{1024, 2, 2};
+  }
   if (Io::kVec == 4) return {1024, 4, 2};
   if (Io::kVec == 16) return kMode == AxpyMode::kTwo ? AxpyShape{640, 2, 2} : AxpyShape{768, 2, 1};
   return kMode == AxpyMode::kOne   ? AxpyShape{1024, 2, 2}
@@ -439,9 +487,7 @@ __device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thre
   // FP8 storage, with twice the blocks per vector, that spills)
   constexpr bool kWide = kMode == AxpyMode::kOne && V <= 8;
   const uint32_t j_hi = static_cast<uint32_t>(j_thread >> 32);
-  const auto gen1 = sched_gen<kWide>(a.s1, j_hi);
-  const auto gen2 = sched_gen<kWide>(a.s2, j_hi);
-  const float s1 = a.scale1 * inv, s2 = a.scale2 * inv;
+  const AxpyGens<kMode, kWide> gens(a, j_hi);
   Round0 p0 = philox_round0<kWide>(static_cast<uint32_t>(j_thread));
   uint4 v[D];
 #pragma unroll
@@ -458,11 +504,11 @@ __device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thre
 #pragma unroll
       for (int b = 0; b < NB; ++b) r0[b] = round0_step(p0, static_cast<uint32_t>(u * (kStride / 4) + b));
       axpy_values<Io, kMode, V>(
-          [&](bool second, uint4 (&x)[NB]) {
+          [&](int i, uint4 (&x)[NB]) {
 #pragma unroll
-            for (int b = 0; b < NB; ++b) x[b] = second ? gen2.block_r0(r0[b]) : gen1.block_r0(r0[b]);
+            for (int b = 0; b < NB; ++b) x[b] = gens.words(a, i, r0[b]);
           },
-          s1, s2, f);
+          a, inv, f);
       *reinterpret_cast<uint4*>(p + u * kStride) = Io::pack(f);
     }
     if (--tiles == 0) return;
@@ -488,17 +534,16 @@ __device__ __forceinline__ void axpy_units(const SegDesc* __restrict__ segs,
     Io::unpack_unit(raw, f);
     // a unit's two blocks start at an even one, so they share the high word
     const uint32_t j_hi = static_cast<uint32_t>(r.j0 >> 32);
-    const auto gen1 = sched_gen<false>(a.s1, j_hi);
-    const auto gen2 = sched_gen<false>(a.s2, j_hi);
+    const AxpyGens<kMode, false> gens(a, j_hi);
     Round0 r0[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) r0[b] = philox_round0<false>(static_cast<uint32_t>(r.j0 + b));
     axpy_values<Io, kMode, kUnit>(
-        [&](bool second, uint4 (&x)[NB]) {
+        [&](int i, uint4 (&x)[NB]) {
 #pragma unroll
-          for (int b = 0; b < NB; ++b) x[b] = second ? gen2.block_r0(r0[b]) : gen1.block_r0(r0[b]);
+          for (int b = 0; b < NB; ++b) x[b] = gens.words(a, i, r0[b]);
         },
-        a.scale1 * r.inv, a.scale2 * r.inv, f);
+        a, r.inv, f);
     Io::store_unit(r.p, r.rem, Io::pack_unit(f));
   }
 }
@@ -1049,13 +1094,7 @@ cudaError_t launch_axpy_io(const PlanView& plan, const AxpyArgs& a, cudaStream_t
 }
 
 template <AxpyMode kMode>
-cudaError_t launch_axpy(const PlanView& plan, uint64_t seed, float scale, uint64_t seed2,
-                        float scale2, cudaStream_t stream) {
-  AxpyArgs a;
-  a.s1 = philox_sched(seed);
-  a.s2 = philox_sched(seed2);
-  a.scale1 = scale;
-  a.scale2 = scale2;
+cudaError_t launch_axpy(const PlanView& plan, const AxpyArgs& a, cudaStream_t stream) {
   if (plan.dtype == ES_BF16) return launch_axpy_io<Bf16Io, kMode>(plan, a, stream);
   if (plan.dtype == ES_FP8_E4M3) return launch_axpy_io<Fp8Io, kMode>(plan, a, stream);
   return launch_axpy_io<F32Io, kMode>(plan, a, stream);
@@ -1065,14 +1104,21 @@ cudaError_t launch_axpy(const PlanView& plan, uint64_t seed, float scale, uint64
 
 cudaError_t launch_axpy_noise(const PlanView& plan, uint64_t seed, float scale,
                               cudaStream_t stream) {
-  return launch_axpy<AxpyMode::kOne>(plan, seed, scale, 0u, 0.0f, stream);
+  AxpyArgs a{};
+  a.seed[0] = philox_sched(seed);
+  a.scale[0] = scale;
+  return launch_axpy<AxpyMode::kOne>(plan, a, stream);
 }
 
 cudaError_t launch_axpy_noise2(const PlanView& plan, uint64_t seed, float scale, uint64_t seed2,
                                float scale2, cudaStream_t stream) {
-  if (seed == seed2)
-    return launch_axpy<AxpyMode::kFlip>(plan, seed, scale, seed2, scale2, stream);
-  return launch_axpy<AxpyMode::kTwo>(plan, seed, scale, seed2, scale2, stream);
+  AxpyArgs a{};
+  a.seed[0] = philox_sched(seed);
+  a.seed[1] = philox_sched(seed2);
+  a.scale[0] = scale;
+  a.scale[1] = scale2;
+  return seed == seed2 ? launch_axpy<AxpyMode::kFlip>(plan, a, stream)
+                       : launch_axpy<AxpyMode::kTwo>(plan, a, stream);
 }
 
 template <class Io, bool kSingle, bool kPerturb>
@@ -1092,6 +1138,19 @@ cudaError_t launch_update_dtype(const PlanView& plan, const UpdateArgs& args, cu
 }
 
 cudaError_t launch_update(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
+  if (args.n_gen == 1 && !args.perturb && args.n <= kMaxSum) {
+    AxpyArgs a{};
+    for (int i = 0; i < args.n; ++i) {
+      a.seed[i] = philox_sched(static_cast<uint64_t>(args.key[i][1]) << 32 | args.key[i][0]);
+      a.scale[i] = args.coeff[i];
+    }
+    switch (args.n) {
+      case 1: return launch_axpy<AxpyMode::kSum1>(plan, a, stream);
+      case 2: return launch_axpy<AxpyMode::kSum2>(plan, a, stream);
+      case 3: return launch_axpy<AxpyMode::kSum3>(plan, a, stream);
+      default: return launch_axpy<AxpyMode::kSum4>(plan, a, stream);
+    }
+  }
   if (plan.dtype == ES_BF16) return launch_update_dtype<Bf16Io>(plan, args, stream);
   if (plan.dtype == ES_FP8_E4M3) return launch_update_dtype<Fp8Io>(plan, args, stream);
   return launch_update_dtype<F32Io>(plan, args, stream);
