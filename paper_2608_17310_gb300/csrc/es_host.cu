@@ -428,19 +428,23 @@ es_status_t es_replay(es_plan_t plan, const uint64_t* seeds, const float* coeffs
   es_status_t st = check_plan_device(plan);
   if (st != ES_OK) return st;
   // Launches break only between generations, so the roundings are those of
-  // one es_update per generation. Small generations share a pass over theta
-  // (fewer passes: measured 5 % faster at 2 seeds per generation, 15 % at 1);
-  // a generation of kOwnLaunch or more non-zero seeds gets a launch of its own
-  // through the single-generation kernel, which runs such generations faster
-  // (measured 2-3 % at 6 to 16 seeds). Both orders give the same bits.
-  constexpr int kOwnLaunch = 4;
+  // one es_update per generation, whichever way they are grouped. On small sets
+  // generations share a pass over theta, which saves a launch each; from kOwnPass
+  // parameters on a generation gets a pass of its own, through the
+  // single-generation kernels, which run faster than the shared pass's rounding
+  // between generations. Not so one fp32 seed, bound by HBM alone. Measured, us
+  // for 8 generations, shared / own: 2 bf16 seeds over 2^20 parameters 16.5 / 31.0,
+  // 2^24 203 / 217, 2^26 800 / 785, 2^28 3181 / 2993; 1 fp32 seed 2^28 1686 / 2629.
+  constexpr uint64_t kOwnPass = uint64_t{1} << 25;
+  const bool large = plan->numel >= kOwnPass;
+  const int own_from = plan->dtype == ES_FP32 ? 2 : 1;
   esopt::UpdateArgs args;
   start_update(args);
   uint64_t off = 0;
   for (int g = 0; g < generations; ++g) {
     int nonzero = 0;
     for (int i = 0; i < counts[g]; ++i) nonzero += coeffs[off + i] != 0.0f;
-    const bool own = nonzero >= kOwnLaunch;
+    const bool own = large && nonzero >= own_from;
     if (nonzero > 0 && args.n_gen > 0 &&
         (own || args.n + nonzero > ES_MAX_SEEDS || args.n_gen == esopt::kMaxGenerations)) {
       st = launch_update_args(plan, args, stream, "es_replay");

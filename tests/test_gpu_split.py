@@ -122,3 +122,27 @@ def test_noise_fill_alignments(es, oracle, lead):
             torch.cuda.synchronize()
             assert torch.equal(out[4 + lead:4 + lead + n], whole[skip:skip + n]), (skip, n)
             assert torch.all(out[:4 + lead] == 7.0) and torch.all(out[4 + lead + n:] == 7.0)
+
+
+# On both sides of the size from which a replayed generation gets a pass of its
+# own: bit-identical to one es_update per generation.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("numel", [2**25 - 8, 2**25])
+def test_replay_passes(es, dtype, numel):
+    a = torch.empty(numel, device="cuda").normal_(0.0, 0.02)
+    a = a.to(torch.bfloat16) if dtype == "bf16" else a
+    b = a.clone()
+    counts = [1, 1, 2, 6, 1, 3, 140, 1, 2]
+    seeds = np.arange(1, sum(counts) + 1, dtype=np.uint64)
+    coeffs = np.linspace(-1e-3, 1e-3, seeds.size).astype(np.float32)
+    coeffs[2:4] = [0.0, 1e-3]  # generation 2 has one non-zero seed
+    plan_a, plan_b = es.plan_from_tensors([a]), es.plan_from_tensors([b])
+    es.es_replay(plan_a, seeds, coeffs, counts)
+    at = 0
+    for n in counts:
+        es.es_update(plan_b, seeds[at:at + n], coeffs[at:at + n])
+        at += n
+    torch.cuda.synchronize()
+    assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+    plan_a.close()
+    plan_b.close()
