@@ -71,6 +71,10 @@ def _load() -> ctypes.CDLL:
     vp, u64, f32, f64, i32 = (ctypes.c_void_p, ctypes.c_uint64, ctypes.c_float,
                               ctypes.c_double, ctypes.c_int)
     P = ctypes.POINTER
+    # numeric arrays go by address (_addr): a typed ctypes pointer takes 2-3 us to
+    # build, and small calls are bound by their host time (es_update of a set that
+    # one SM holds: 14.5 us a call with typed pointers and a Stream object, 6.2 us so)
+    arr = vp
     sigs = {
         "es_plan_create": (i32, [P(es_segment_t), i32, i32, P(vp)]),
         "es_plan_create_scaled": (i32, [P(es_segment_t), P(f32), i32, i32, P(vp)]),
@@ -83,13 +87,13 @@ def _load() -> ctypes.CDLL:
         "es_perturb": (i32, [vp, u64, f32, vp]),
         "es_restore": (i32, [vp, u64, f32, vp]),
         "es_restore_perturb": (i32, [vp, u64, f32, u64, f32, vp]),
-        "es_update": (i32, [vp, P(u64), P(f32), i32, vp]),
-        "es_update_perturb": (i32, [vp, P(u64), P(f32), i32, u64, f32, vp]),
-        "es_replay": (i32, [vp, P(u64), P(f32), P(i32), i32, vp]),
-        "es_normalize_rewards": (i32, [P(f64), i32, f64, P(f64)]),
+        "es_update": (i32, [vp, arr, arr, i32, vp]),
+        "es_update_perturb": (i32, [vp, arr, arr, i32, u64, f32, vp]),
+        "es_replay": (i32, [vp, arr, arr, arr, i32, vp]),
+        "es_normalize_rewards": (i32, [arr, i32, f64, arr]),
         "es_sigma_cosine": (f64, [f64, f64, i32, i32]),
-        "es_update_coeffs": (i32, [P(f64), i32, f64, f64, i32, P(f32)]),
-        "es_fold_antithetic": (i32, [P(f64), P(f64), i32, f64, f64, i32, P(f32)]),
+        "es_update_coeffs": (i32, [arr, i32, f64, f64, i32, arr]),
+        "es_fold_antithetic": (i32, [arr, arr, i32, f64, f64, i32, arr]),
         "es_perturb_noalloc": (i32, [P(es_segment_t), i32, i32, u64, f32, vp]),
         "es_status_string": (ctypes.c_char_p, [i32]),
         "es_last_error": (ctypes.c_char_p, []),
@@ -123,11 +127,21 @@ def _check(status: int, func: str) -> None:
         raise EsError(status, func, es_last_error())
 
 
+def _current_stream(torch) -> int:
+    # torch.cuda.current_stream() builds a Stream object (2.9 us); its raw form,
+    # where this torch has it, gives the same handle in 0.1 us
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch._C._cuda_getDevice())
+
+
 def _stream(stream) -> int:
     if stream is None:
         torch = sys.modules.get("torch")
-        if torch is not None and torch.cuda.is_available() and torch.cuda.is_initialized():
-            return torch.cuda.current_stream().cuda_stream
+        # an initialised torch.cuda is an available one
+        if torch is not None and torch.cuda.is_initialized():
+            return _current_stream(torch)
         return 0
     if isinstance(stream, int):
         return stream
@@ -138,6 +152,10 @@ def _ptr(buf) -> int:
     if isinstance(buf, int):
         return buf
     return int(buf.data_ptr())
+
+
+def _addr(a: np.ndarray) -> int:
+    return a.ctypes.data
 
 
 def _f64(a) -> np.ndarray:
@@ -203,7 +221,8 @@ def es_assign_index_bases(segments: Sequence[Segment]) -> int:
 def es_plan_create(segments: Sequence[Segment], dtype: int, keepalive: Iterable = ()) -> Plan:
     arr = _seg_array(segments)
     handle = ctypes.c_void_p()
-    _check(_load().es_plan_create(arr, len(segments), dtype, ctypes.byref(handle)),
+    _check(_load().es_plan_create(arr, len(segments), dtype,
+        ctypes.byref(handle)),
            "es_plan_create")
     return Plan(handle.value, int(_load().es_plan_numel(handle)), dtype, keepalive)
 
@@ -216,8 +235,9 @@ def es_plan_create_scaled(segments: Sequence[Segment], scales, dtype: int,
     if sc.size != len(segments):
         raise ValueError("one scale per segment")
     handle = ctypes.c_void_p()
-    _check(_load().es_plan_create_scaled(arr, sc.ctypes.data_as(ctypes.POINTER(ctypes.c_float)),
-                                         len(segments), dtype, ctypes.byref(handle)),
+    _check(_load().es_plan_create_scaled(
+        arr, sc.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), len(segments), dtype,
+        ctypes.byref(handle)),
            "es_plan_create_scaled")
     return Plan(handle.value, int(_load().es_plan_numel(handle)), dtype, keepalive, sc)
 
@@ -296,9 +316,8 @@ def es_update(plan: Plan, seeds, coeffs, stream=None) -> None:
     c = np.ascontiguousarray(coeffs, dtype=np.float32)
     if s.size != c.size:
         raise ValueError("seeds and coeffs differ in length")
-    _check(_load().es_update(plan.handle, s.ctypes.data_as(ctypes.POINTER(ctypes.c_uint64)),
-                             c.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), s.size,
-                             _stream(stream)), "es_update")
+    _check(_load().es_update(plan.handle, _addr(s), _addr(c), s.size, _stream(stream)),
+           "es_update")
 
 
 def es_perturb_noalloc(segments: Sequence[Segment], dtype: int, seed: int, sigma: float,
@@ -316,9 +335,8 @@ def es_update_perturb(plan: Plan, seeds, coeffs, next_seed: int, sigma_next: flo
     c = np.ascontiguousarray(coeffs, dtype=np.float32)
     if s.size != c.size:
         raise ValueError("seeds and coeffs differ in length")
-    _check(_load().es_update_perturb(plan.handle, s.ctypes.data_as(ctypes.POINTER(ctypes.c_uint64)),
-                                     c.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), s.size,
-                                     next_seed, sigma_next, _stream(stream)), "es_update_perturb")
+    _check(_load().es_update_perturb(plan.handle, _addr(s), _addr(c), s.size, next_seed,
+                                     sigma_next, _stream(stream)), "es_update_perturb")
 
 
 def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
@@ -328,10 +346,8 @@ def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
     n = np.ascontiguousarray(counts, dtype=np.int32)
     if s.size != c.size or int(n.sum()) != s.size:
         raise ValueError("seeds, coeffs and counts do not agree")
-    _check(_load().es_replay(plan.handle, s.ctypes.data_as(ctypes.POINTER(ctypes.c_uint64)),
-                             c.ctypes.data_as(ctypes.POINTER(ctypes.c_float)),
-                             n.ctypes.data_as(ctypes.POINTER(ctypes.c_int)), n.size,
-                             _stream(stream)), "es_replay")
+    _check(_load().es_replay(plan.handle, _addr(s), _addr(c), _addr(n), n.size, _stream(stream)),
+           "es_replay")
 
 
 # --- host-side generation control ---------------------------------------------------
@@ -339,9 +355,8 @@ def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
 def es_normalize_rewards(rewards, eps_z: float = 1e-8) -> np.ndarray:
     r = _f64(rewards)
     out = np.empty_like(r)
-    P = ctypes.POINTER(ctypes.c_double)
-    _check(_load().es_normalize_rewards(r.ctypes.data_as(P), r.size, eps_z,
-                                        out.ctypes.data_as(P)), "es_normalize_rewards")
+    _check(_load().es_normalize_rewards(_addr(r), r.size, eps_z, _addr(out)),
+           "es_normalize_rewards")
     return out
 
 
@@ -352,9 +367,7 @@ def es_sigma_cosine(sigma0: float, sigmaT: float, t: int, T: int) -> float:
 def es_update_coeffs(rhat, alpha: float, sigma: float, mode: int = ES_SCALE_PAPER) -> np.ndarray:
     r = _f64(rhat)
     out = np.empty(r.size, dtype=np.float32)
-    _check(_load().es_update_coeffs(r.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), r.size,
-                                    alpha, sigma, mode,
-                                    out.ctypes.data_as(ctypes.POINTER(ctypes.c_float))),
+    _check(_load().es_update_coeffs(_addr(r), r.size, alpha, sigma, mode, _addr(out)),
            "es_update_coeffs")
     return out
 
@@ -365,9 +378,6 @@ def es_fold_antithetic(rhat_pos, rhat_neg, alpha: float, sigma: float,
     if p.size != m.size:
         raise ValueError("rhat_pos and rhat_neg differ in length")
     out = np.empty(p.size, dtype=np.float32)
-    P = ctypes.POINTER(ctypes.c_double)
-    _check(_load().es_fold_antithetic(p.ctypes.data_as(P), m.ctypes.data_as(P), p.size, alpha,
-                                      sigma, mode,
-                                      out.ctypes.data_as(ctypes.POINTER(ctypes.c_float))),
+    _check(_load().es_fold_antithetic(_addr(p), _addr(m), p.size, alpha, sigma, mode, _addr(out)),
            "es_fold_antithetic")
     return out
