@@ -70,7 +70,8 @@ es_status_t check_device_buffer(const void* p, const char* what) {
 }
 
 esopt::PlanView view(const es_plan* plan) {
-  return esopt::PlanView{plan->d_segs, plan->nseg, plan->granules, plan->dtype, plan->d_inv_scale};
+  return esopt::PlanView{plan->d_segs, plan->nseg, plan->granules, plan->dtype, plan->d_inv_scale,
+                         true};
 }
 
 es_status_t check_update_inputs(es_plan_t plan, const uint64_t* seeds, const float* coeffs, int n,

@@ -61,6 +61,9 @@ struct PlanView {
   es_dtype_t dtype;
   // ES_FP8_E4M3: device array of 1 / scale per segment; NULL otherwise
   const float* inv_scale;
+  // whether a launch may read the table before earlier work in its stream has
+  // ended: true of a plan's own table, false of one that the stream itself copies
+  bool early;
 };
 
 // Kernel launchers (es_kernels.cu). Each returns the launch's cudaError_t.

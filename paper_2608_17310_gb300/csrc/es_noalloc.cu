@@ -186,7 +186,7 @@ extern "C" es_status_t es_perturb_noalloc(const es_segment_t* segs, int nseg, es
   err = cudaMemcpyAsync(d_table, table, (static_cast<size_t>(nseg) + 1) * sizeof(SegDesc),
                         cudaMemcpyHostToDevice, s);
   if (err != cudaSuccess) return reject(ES_ERR_CUDA, "es_perturb_noalloc: copy of the segment table failed");
-  err = esopt::launch_axpy_noise(esopt::PlanView{d_table, nseg, granules, dtype, nullptr}, seed, sigma, s);
+  err = esopt::launch_axpy_noise(esopt::PlanView{d_table, nseg, granules, dtype, nullptr, false}, seed, sigma, s);
   if (err != cudaSuccess) return reject(ES_ERR_CUDA, "es_perturb_noalloc: kernel launch failed");
   return esopt::record_status(ES_OK, "");
 }

@@ -146,3 +146,58 @@ def test_replay_passes(es, dtype, numel):
     assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
     plan_a.close()
     plan_b.close()
+
+
+# A launch may start before the kernel before it has ended. Behind every kind of
+# work that a stream can hold (kernels of its own kind, other kernels, copies,
+# fills, a join of two streams), eager and captured into a graph, the result is that
+# of the same calls with the device synchronised in between.
+@pytest.mark.parametrize("numel", [1000, 1 << 16, 3_000_001])
+def test_launches_behind_other_work(es, numel):
+    a = torch.empty(numel, device="cuda").normal_(0.0, 0.02)
+    source, host = torch.randn(numel, device="cuda"), torch.randn(numel).pin_memory()
+    start = a.clone()
+    plan = es.plan_from_tensors([a])
+    other = torch.empty(numel, device="cuda")
+    seeds, coeffs = np.arange(6, dtype=np.uint64), np.full(6, 1e-3, dtype=np.float32)
+    side = torch.cuda.Stream()
+
+    def calls(wait):
+        out = []
+        for before in (lambda: a.copy_(start), lambda: a.copy_(host, non_blocking=True),
+                       lambda: a.zero_(), lambda: a.add_(source),
+                       lambda: es.es_noise_fill(5, 0, numel, a), lambda: fork()):
+            before()
+            wait()
+            es.es_perturb(plan, 3, 1e-3)
+            wait()
+            es.es_restore_perturb(plan, 3, 1e-3, 4, 1e-3)
+            wait()
+            es.es_update(plan, seeds, coeffs)
+            wait()
+            es.es_update(plan, seeds[:2], coeffs[:2])
+            wait()
+            out.append(a.clone())
+            wait()
+        return out
+
+    def fork():
+        here = torch.cuda.current_stream()
+        side.wait_stream(here)
+        with torch.cuda.stream(side):
+            es.es_noise_fill(6, 0, numel, other)
+        a.mul_(0.5)
+        here.wait_stream(side)
+
+    want = calls(torch.cuda.synchronize)
+    for got in (calls(lambda: None), calls(lambda: None)):
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(want, got))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = calls(lambda: None)
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(want, got))
+    plan.close()
