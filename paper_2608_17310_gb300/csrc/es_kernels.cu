@@ -74,6 +74,9 @@ struct Bf16Io {
       if (k < rem) p[k] = static_cast<uint16_t>(w[k >> 1] >> (16 * (k & 1)));
   }
   __device__ static Raw zero_unit() { return make_uint4(0u, 0u, 0u, 0u); }
+  // one element: its value, the stored form of a value, and that form's value
+  __device__ static float value(uint16_t h) { return __uint_as_float(static_cast<uint32_t>(h) << 16); }
+  __device__ static uint16_t store(float f) { return static_cast<uint16_t>(pack2(f, 0.0f)); }
   __device__ static void unpack_unit(const Raw& v, float (&f)[kUnit]) { unpack(v, f); }
   __device__ static Raw pack_unit(const float (&f)[kUnit]) { return pack(f); }
 };
@@ -95,6 +98,8 @@ struct F32Io {
   struct Raw {
     uint4 lo, hi;
   };
+  __device__ static float value(float f) { return f; }
+  __device__ static float store(float f) { return f; }
   __device__ static Raw load_unit(const float* p, int rem) {
     if (rem == kUnit) {
       const uint4* q = reinterpret_cast<const uint4*>(p);
@@ -177,6 +182,8 @@ struct Fp8Io {
     }
   }
   using Raw = uint2;
+  __device__ static float value(uint8_t c) { return dec2(c).x; }
+  __device__ static uint8_t store(float f) { return static_cast<uint8_t>(enc2(f, 0.0f)); }
   __device__ static Raw load_unit(const uint8_t* p, int rem) {
     if (rem == kUnit) return *reinterpret_cast<const uint2*>(p);
     uint32_t w[2] = {0u, 0u};
@@ -398,27 +405,34 @@ struct AxpyArgs {
 template <class Io, AxpyMode kMode, int V, class Words>
 __device__ __forceinline__ void axpy_values(const Words& words, const AxpyArgs& a, float inv,
                                             float (&f)[V]) {
+  constexpr int kSeeds = axpy_seeds(kMode);
   uint4 x[V / 4];
+  words(0, x);
   if constexpr (axpy_is_sum(kMode)) {
     float acc[V];
 #pragma unroll
     for (int k = 0; k < V; ++k) acc[k] = 0.0f;
+    // each seed's words before the transform of the one before (2 % faster than
+    // after it; the two-step pass does not gain from it)
 #pragma unroll
-    for (int i = 0; i < axpy_seeds(kMode); ++i) {
-      words(i, x);
+    for (int i = 0; i < kSeeds; ++i) {
+      uint4 y[V / 4];
+      if (i + 1 < kSeeds) words(i + 1, y);
       add_scaled_noise<V>(x, a.scale[i], acc);
+      if (i + 1 < kSeeds) {
+#pragma unroll
+        for (int b = 0; b < V / 4; ++b) x[b] = y[b];
+      }
     }
 #pragma unroll
     for (int k = 0; k < V; ++k) f[k] = add_acc<Io>(f[k], acc[k], inv);
   } else if constexpr (kMode == AxpyMode::kFlip) {
-    words(0, x);
     Polar2 pp[V / 4];
     polar_from_words<V / 4>(x, pp);
     apply_noise<V>(pp, a.scale[0] * inv, f);
     Io::round_trip(f);
     apply_noise<V>(pp, a.scale[1] * inv, f);
   } else {
-    words(0, x);
     add_scaled_noise<V>(x, a.scale[0] * inv, f);
     if constexpr (kMode == AxpyMode::kTwo) {
       Io::round_trip(f);
@@ -454,8 +468,8 @@ struct AxpyGens {
 // steps 1217 -> 1094 (1.449e12 Gaussians/s), flip 729 -> 621; fp32 971 -> 962 (6.59 TB/s: HBM),
 // 1366 -> 1077, 976 -> 961; FP8 636 -> 575, 1301 -> 1127, 718 -> 639.
 // The sums replace the seed loop of update_kernel where it is too short for its
-// pipeline: 1 / 2 / 3 / 4 seeds bf16 972 / 1480 / 2035 / 2555 -> 591 / 1094 /
-// 1599 / 2143, fp32 1125 / 1642 / 2253 / 2866 -> 962 / 1088 / 1589 / 2145, FP8
+// pipeline: 1 / 2 / 3 / 4 seeds bf16 972 / 1480 / 2035 / 2555 -> 591 / 1078 /
+// 1596 / 2107, fp32 1125 / 1642 / 2253 / 2866 -> 962 / 1088 / 1589 / 2145, FP8
 // 811 / 1392 / 1979 / 2567 -> 602 / 1110 / 1608 / 2113.
 // Thread counts that are no multiple of 128 leave the SM's four schedulers
 // unequal warps and run 10 % slower.
@@ -855,6 +869,107 @@ update_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restric
   let_next_start();
 }
 
+// The update of a small set, which leaves most of the GPU's threads without an
+// element: the seeds are spread over the warps too. A CTA takes 8 granules (32
+// Philox blocks, one per lane) and its warps one seed each at a time; the
+// polar forms, scaled, go through shared memory to four of the warps, one per
+// element of a block, which add them up in ascending seed order with the same
+// operations as update_unit, so the values are the same bits. What bounds it is
+// latency: n / kWarps rounds of one block's generation instead of n of two blocks'.
+// 65,536 fp32 parameters, us in a graph (update_unit's or the sums' pass -> this):
+// 1 seed 1.7 -> 1.6, 8 seeds 3.0 -> 2.1, 32 seeds 6.9 -> 5.8, 128 seeds 21.9 -> 20.0;
+// 1024 parameters 32 seeds 6.8 -> 2.5. It generates one block per thread where
+// update_unit overlaps two, so it loses once the GPU is full: 98,304 parameters, 8
+// seeds even, 128 seeds 22.2 -> 29.5. kSplitMaxGranules lies where 128 seeds break
+// even. A CTA of 32 warps, 32 seeds at a time, is the better one while every CTA
+// has an SM to itself (19,000 parameters, 128 seeds 12.6 with 8 warps -> 9.2; 65,536: 20.4 ->
+// 24.0).
+constexpr uint64_t kSplitMaxGranules = 4352;
+constexpr uint64_t kSplitWideGranules = 152 * 8;
+constexpr int kSplitSeeds = 128;
+struct SplitArgs {
+  int n, n_gen, perturb;  // as UpdateArgs
+  float pscale;
+  uint32_t pkey[2];
+  uint8_t gen_end[kSplitSeeds];
+  uint32_t key[kSplitSeeds][2];
+  float coeff[kSplitSeeds];
+};
+constexpr int kSplitGranules = 32 * 4 / kGranule;
+// One warp's scaled polar forms: -(c r) of both pairs, then cos and sin of each.
+using SplitForms = float[6][32];
+
+template <class Io, int kWarps>
+__global__ void __launch_bounds__(32 * kWarps)
+update_split_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
+                    uint64_t granules, const __grid_constant__ SplitArgs args) {
+  __shared__ SplitForms s_forms[2][kWarps];
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const uint64_t first = blockIdx.x * static_cast<uint64_t>(kSplitGranules);
+  const uint64_t end = first + kSplitGranules < granules ? first + kSplitGranules : granules;
+  // the lane's block: 4 elements at e in its segment
+  const int seg0 = search_segment(segs, 0, nseg, first);
+  const int seg1 = search_segment(segs, seg0, nseg, end - 1);
+  const uint64_t mine = first + lane / 4 < end ? first + lane / 4 : end - 1;
+  const int seg = segment_between(segs, seg0, seg1, mine);
+  const SegDesc d = segs[seg];
+  const uint64_t e = (mine - d.granule_begin) * kGranule + lane % 4 * 4;
+  const float inv = Io::kScaled ? inv_scale[seg] : 1.0f;
+  const uint64_t j = (d.index_base + e) >> 2;
+  // warps 0 .. 3 own element `warp` of each block
+  const bool owner = warp < 4 && first + lane / 4 < end && e + warp < d.numel;
+  typename Io::Scalar* const p = static_cast<typename Io::Scalar*>(d.data) + e + warp;
+  float theta = 0.0f, acc = 0.0f;
+  int g = 0;
+  const int items = args.n + args.perturb;  // the perturb comes last
+#pragma unroll 1
+  for (int i0 = 0, buf = 0; i0 < items; i0 += kWarps, buf ^= 1) {
+    const int i = i0 + warp;
+    if (i < items) {
+      const bool last = i == args.n;
+      const PhiloxKey key = last ? PhiloxKey{args.pkey[0], args.pkey[1]}
+                                 : PhiloxKey{args.key[i][0], args.key[i][1]};
+      const float scale = last ? args.pscale * inv : args.coeff[i];
+      const uint4 x[1] = {philox_block(j, key)};
+      Polar2 pp[1];
+      polar_from_words<1>(x, pp);
+      const float2 sr = __fmul2_rn(make_float2(-scale, -scale), pp[0].r);
+      SplitForms& f = s_forms[buf][warp];
+      f[0][lane] = sr.x;
+      f[1][lane] = sr.y;
+      f[2][lane] = pp[0].c.x;
+      f[3][lane] = pp[0].s.x;
+      f[4][lane] = pp[0].c.y;
+      f[5][lane] = pp[0].s.y;
+    }
+    if (i0 == 0) {
+      wait_for_previous();
+      if (owner) theta = Io::value(*p);
+    }
+    __syncthreads();
+    if (warp >= 4) continue;
+    const int m = items - i0 < kWarps ? items - i0 : kWarps;
+#pragma unroll 8
+    for (int k = 0; k < kWarps; ++k) {
+      if (k >= m) break;
+      const SplitForms& f = s_forms[buf][k];
+      const float sr = f[warp / 2][lane], t = f[2 + warp][lane];
+      if (i0 + k == args.n) {
+        theta = Io::value(Io::store(fmaf(sr, t, theta)));
+      } else {
+        acc = fmaf(sr, t, acc);
+        if (i0 + k + 1 == args.gen_end[g]) {
+          theta = Io::value(Io::store(add_acc<Io>(theta, acc, inv)));
+          acc = 0.0f;
+          if (g + 1 < args.n_gen) ++g;
+        }
+      }
+    }
+  }
+  if (owner) *p = Io::store(theta);
+  let_next_start();
+}
+
 // es_noise_fill. `out` is cut into aligned 16-byte groups of 4 floats, and group
 // m lies `lead` floats before out[4m]; its values come from one Philox block
 // (kShift 0) or from the last 4 - kShift values of one block and the first
@@ -1177,7 +1292,43 @@ cudaError_t launch_update_dtype(const PlanView& plan, const UpdateArgs& args, cu
                       : launch_update_io<Io, true, false>(plan, args, stream);
 }
 
+template <class Io, int kWarps>
+cudaError_t launch_split_warps(const PlanView& plan, const SplitArgs& args, cudaStream_t stream) {
+  return launch_early(update_split_kernel<Io, kWarps>,
+                      static_cast<int>((plan.granules + kSplitGranules - 1) / kSplitGranules),
+                      32 * kWarps, plan.early, stream, plan.segs, plan.nseg, plan.inv_scale,
+                      plan.granules, args);
+}
+
+template <class Io>
+cudaError_t launch_split_io(const PlanView& plan, const SplitArgs& args, cudaStream_t stream) {
+  if (args.n + args.perturb > 8 && plan.granules <= kSplitWideGranules)
+    return launch_split_warps<Io, 32>(plan, args, stream);
+  return launch_split_warps<Io, 8>(plan, args, stream);
+}
+
+cudaError_t launch_update_split(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
+  SplitArgs a;
+  a.n = args.n;
+  a.n_gen = args.n_gen;
+  a.perturb = args.perturb;
+  a.pscale = args.pscale;
+  a.pkey[0] = args.pkey[0];
+  a.pkey[1] = args.pkey[1];
+  for (int g = 0; g < args.n_gen; ++g) a.gen_end[g] = static_cast<uint8_t>(args.gen_end[g]);
+  for (int i = 0; i < args.n; ++i) {
+    a.key[i][0] = args.key[i][0];
+    a.key[i][1] = args.key[i][1];
+    a.coeff[i] = args.coeff[i];
+  }
+  if (plan.dtype == ES_BF16) return launch_split_io<Bf16Io>(plan, a, stream);
+  if (plan.dtype == ES_FP8_E4M3) return launch_split_io<Fp8Io>(plan, a, stream);
+  return launch_split_io<F32Io>(plan, a, stream);
+}
+
 cudaError_t launch_update(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
+  if (args.n <= kSplitSeeds && plan.granules <= kSplitMaxGranules)
+    return launch_update_split(plan, args, stream);
   if (args.n_gen == 1 && !args.perturb && args.n <= kMaxSum) {
     AxpyArgs a{};
     for (int i = 0; i < args.n; ++i) {

@@ -201,3 +201,61 @@ def test_launches_behind_other_work(es, numel):
     torch.cuda.synchronize()
     assert all(torch.equal(x, y) for x, y in zip(want, got))
     plan.close()
+
+
+# The update of a small set, whose seeds are spread over warps: the same bits as
+# in a plan that a further, larger tensor takes out of that range, and equal to the
+# oracle; counts at the edges of a round of 8 and of 32 seeds, sets on both sides of
+# the change between them and at the largest, ragged segments and a segment
+# across the change of the high counter word.
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "fp8"])
+@pytest.mark.parametrize("numels", [[1], [7, 1, 130, 16], [19_456], [19_457, 3], [5_000, 64_000]])
+def test_small_set_update(es, oracle, dtype, numels):
+    rng = np.random.default_rng(sum(numels))
+    if dtype == "fp8":
+        tensors = [torch.from_numpy(rng.integers(0, 120, size=n).astype(np.uint8)).cuda()
+                   for n in numels]
+        scales = [2.0**-9 * (k + 1) for k in range(len(numels))]
+        more = torch.zeros(1 << 20, dtype=torch.uint8, device="cuda")
+    else:
+        tensors, scales = make_params(dtype, numels, seed=5), None
+        more = torch.zeros(1 << 20, dtype=tensors[0].dtype, device="cuda")
+    twins = [t.clone() for t in tensors]
+    bases = [2**34 - 8 * (numels[0] // 16)]
+    for n in numels[:-1]:
+        bases.append((bases[-1] + n + 7) // 8 * 8 + 16)
+    small = es.plan_from_tensors(tensors, bases, scales)
+    large = es.plan_from_tensors(twins + [more], bases + [2**40], scales and scales + [1.0])
+
+    def same(what):
+        torch.cuda.synchronize()
+        for x, y in zip(tensors, twins):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8)), what
+
+    for n in (1, 4, 5, 7, 8, 9, 16, 31, 32, 33, 127, 128, 129):
+        seeds = rng.integers(0, 2**63, size=n).astype(np.uint64)
+        coeffs = (1e-3 * rng.standard_normal(n)).astype(np.float32)
+        before = [t.cpu().numpy() if dtype == "fp8" else host_values(t) for t in tensors]
+        for p in (small, large):
+            es.es_update(p, seeds, coeffs)
+        same(n)
+        for k, t in enumerate(tensors if n in (5, 33) else []):
+            g = np.arange(bases[k], bases[k] + numels[k], dtype=np.uint64)
+            tol = noise_abs_tol([oracle.noise_at(int(s), g) for s in seeds], coeffs)
+            if dtype == "fp8":
+                from test_gpu_fp8 import assert_e4m3_close
+                assert_e4m3_close(t.cpu().numpy(), oracle.update(before[k], g, seeds, coeffs, "e4m3",
+                                                                 scales[k]), n, tol / scales[k])
+            else:
+                compare(dtype, host_values(t), oracle.update(before[k], g, seeds, coeffs, dtype),
+                        f"{n} seeds", tol)
+        for p in (small, large):
+            es.es_update_perturb(p, seeds, coeffs, 77, 1e-3)
+        same((n, "perturb"))
+        counts = [n - n // 3, n // 3] if n >= 3 else [n]
+        for p in (small, large):
+            es.es_replay(p, seeds, coeffs, counts)
+            es.es_replay(p, seeds, coeffs, [1] * n)
+        same((n, "replay"))
+    small.close()
+    large.close()
