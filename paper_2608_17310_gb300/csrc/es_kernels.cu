@@ -362,16 +362,14 @@ struct UnitRef {
 };
 
 template <class Io>
-__device__ __forceinline__ UnitRef<Io> unit_ref(const SegDesc* __restrict__ segs,
-                                                const float* __restrict__ inv_scale, int seg,
+__device__ __forceinline__ UnitRef<Io> unit_ref(const SegDesc& d, float inv,
                                                 uint64_t unit) {
-  const SegDesc d = segs[seg];
   const uint64_t e = (unit - d.granule_begin * kUnitsPerGranule) * kUnit;
   UnitRef<Io> r;
   r.rem = e >= d.numel ? 0 : d.numel - e < kUnit ? static_cast<int>(d.numel - e) : kUnit;
   r.p = static_cast<typename Io::Scalar*>(d.data) + e;
   r.j0 = (d.index_base + e) >> 2;
-  r.inv = Io::kScaled ? inv_scale[seg] : 1.0f;
+  r.inv = inv;
   return r;
 }
 
@@ -545,35 +543,27 @@ __device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thre
   }
 }
 
-// Units q .. stop - 1, which lie in segments first .. last: one unit per
-// thread at a time, its segment found by the thread itself.
+// One unit of the calling thread.
 template <class Io, AxpyMode kMode>
-__device__ __forceinline__ void axpy_units(const SegDesc* __restrict__ segs,
-                                           const float* __restrict__ inv_scale, int first, int last,
-                                           uint64_t q, uint64_t stop, const AxpyArgs& a) {
+__device__ __forceinline__ void axpy_unit(const UnitRef<Io>& r, const AxpyArgs& a) {
   constexpr int NB = kUnit / 4;
-#pragma unroll 1
-  for (q += threadIdx.x; q < stop; q += blockDim.x) {
-    const UnitRef<Io> r = unit_ref<Io>(
-        segs, inv_scale, segment_between(segs, first, last, q / kUnitsPerGranule), q);
-    if (r.rem == 0) continue;
-    const typename Io::Raw raw = Io::load_unit(r.p, r.rem);
-    float f[kUnit];
-    Io::unpack_unit(raw, f);
-    // a unit's two blocks start at an even one, so they share the high word
-    const uint32_t j_hi = static_cast<uint32_t>(r.j0 >> 32);
-    const AxpyGens<kMode, false> gens(a, j_hi);
-    Round0 r0[NB];
+  if (r.rem == 0) return;
+  const typename Io::Raw raw = Io::load_unit(r.p, r.rem);
+  float f[kUnit];
+  Io::unpack_unit(raw, f);
+  // a unit's two blocks start at an even one, so they share the high word
+  const uint32_t j_hi = static_cast<uint32_t>(r.j0 >> 32);
+  const AxpyGens<kMode, false> gens(a, j_hi);
+  Round0 r0[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) r0[b] = philox_round0<false>(static_cast<uint32_t>(r.j0 + b));
-    axpy_values<Io, kMode, kUnit>(
-        [&](int i, uint4 (&x)[NB]) {
+  for (int b = 0; b < NB; ++b) r0[b] = philox_round0<false>(static_cast<uint32_t>(r.j0 + b));
+  axpy_values<Io, kMode, kUnit>(
+      [&](int i, uint4 (&x)[NB]) {
 #pragma unroll
-          for (int b = 0; b < NB; ++b) x[b] = gens.words(a, i, r0[b]);
-        },
-        a, r.inv, f);
-    Io::store_unit(r.p, r.rem, Io::pack_unit(f));
-  }
+        for (int b = 0; b < NB; ++b) x[b] = gens.words(a, i, r0[b]);
+      },
+      a, r.inv, f);
+  Io::store_unit(r.p, r.rem, Io::pack_unit(f));
 }
 
 // theta[g] <- round(theta[g] + scale * eps_seed[g]) over every segment, or the
@@ -581,7 +571,8 @@ __device__ __forceinline__ void axpy_units(const SegDesc* __restrict__ segs,
 // added in units of the segment's scale: scale * inv_scale[segment].
 // A CTA alternates between runs of whole tiles inside one segment (axpy_run)
 // and up to a tile's worth of units wherever a segment, the range or a high
-// counter word ends (axpy_units).
+// counter word ends (axpy_unit; each thread finds its unit's segment). It waits for
+// the kernel before it only when it has read the table.
 template <class Io, AxpyMode kMode>
 __global__ void __launch_bounds__(axpy_shape<Io, kMode>().threads, 1)
 axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
@@ -591,7 +582,6 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
   uint64_t q = range_begin(split) * kUnitsPerGranule;
   const uint64_t end = range_end(split) * kUnitsPerGranule;
   int seg = search_segment(segs, 0, nseg, q / kUnitsPerGranule);
-  wait_for_previous();
   while (q < end) {
     if (q / kUnitsPerGranule >= segs[seg + 1].granule_begin)
       seg = search_segment(segs, seg + 1, nseg, q / kUnitsPerGranule);
@@ -608,6 +598,7 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
       if (tiles > 0) {
         if (tiles > 0x7FFFFFFFu) tiles = 0x7FFFFFFFu;
         const uint64_t mine = threadIdx.x * static_cast<uint64_t>(Io::kVec);
+        wait_for_previous();
         axpy_run<Io, kMode>(static_cast<typename Io::Scalar*>(d.data) + e + mine, (g + mine) >> 2,
                             static_cast<uint32_t>(tiles), a, Io::kScaled ? inv_scale[seg] : 1.0f);
         q += tiles * kTile;
@@ -616,7 +607,28 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
     }
     const uint64_t stop = q + kTile < end ? q + kTile : end;
     const int last = search_segment(segs, seg, nseg, (stop - 1) / kUnitsPerGranule);
-    axpy_units<Io, kMode>(segs, inv_scale, seg, last, q, stop, a);
+    wait_for_previous();
+    // Units of one segment take its entry from registers, which saves a launch
+    // 0.2-0.5 us (2^22 bf16 parameters 5.9 -> 5.5 us); in the bf16 two-step pass
+    // and sums the second loop costs the run above 2 % instead
+    constexpr bool kKeep = Io::kVec != 8 || kMode == AxpyMode::kOne || kMode == AxpyMode::kFlip;
+    bool done = false;
+    if constexpr (kKeep) {
+      if (seg == last) {
+        const float inv = Io::kScaled ? inv_scale[seg] : 1.0f;
+#pragma unroll 1
+        for (uint64_t u = q + threadIdx.x; u < stop; u += blockDim.x)
+          axpy_unit<Io, kMode>(unit_ref<Io>(d, inv, u), a);
+        done = true;
+      }
+    }
+    if (!done) {
+#pragma unroll 1
+      for (uint64_t u = q + threadIdx.x; u < stop; u += blockDim.x) {
+        const int s = segment_between(segs, seg, last, u / kUnitsPerGranule);
+        axpy_unit<Io, kMode>(unit_ref<Io>(segs[s], Io::kScaled ? inv_scale[s] : 1.0f, u), a);
+      }
+    }
     __syncwarp();
     q = stop;
     seg = last;
@@ -813,7 +825,6 @@ update_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restric
   uint64_t q = range_begin(split) * kUnitsPerGranule;
   const uint64_t end = range_end(split) * kUnitsPerGranule;
   int seg = search_segment(segs, 0, nseg, q / kUnitsPerGranule);
-  wait_for_previous();
 #pragma unroll 1
   while (q < end) {
     if (q / kUnitsPerGranule >= segs[seg + 1].granule_begin)
@@ -837,6 +848,8 @@ update_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restric
         Round0 p0[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) p0[b] = philox_round0<false>(j0 + b);
+        ensure_rows<kPerturb>(s_rows, rs, args, 0, j_hi);
+        wait_for_previous();
 #pragma unroll 1
         for (;;) {
           update_unit<Io, true, kSingle, kPerturb>(p, kUnit, inv, j_hi, p0, j_hi, args, s_rows, rs);
@@ -851,13 +864,15 @@ update_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restric
     const uint64_t stop = q + row < end ? q + row : end;
     const int last = search_segment(segs, seg, nseg, (stop - 1) / kUnitsPerGranule);
     const uint64_t mine = q + threadIdx.x < stop ? q + threadIdx.x : stop - 1;
-    const UnitRef<Io> r = unit_ref<Io>(
-        segs, inv_scale, segment_between(segs, seg, last, mine / kUnitsPerGranule), mine);
+    const int s = segment_between(segs, seg, last, mine / kUnitsPerGranule);
+    const UnitRef<Io> r = unit_ref<Io>(segs[s], Io::kScaled ? inv_scale[s] : 1.0f, mine);
     const int rem = q + threadIdx.x < stop ? r.rem : 0;
     Round0 p0[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) p0[b] = philox_round0<false>(static_cast<uint32_t>(r.j0 + b));
     const uint32_t my_hi = static_cast<uint32_t>(r.j0 >> 32);
+    ensure_rows<kPerturb>(s_rows, rs, args, 0, j_hi);
+    wait_for_previous();
     // the staged constants are those of the row's first unit
     if (__syncthreads_and(rem == 0 || my_hi == j_hi))
       update_unit<Io, true, kSingle, kPerturb>(r.p, rem, r.inv, my_hi, p0, j_hi, args, s_rows, rs);
