@@ -19,15 +19,31 @@
 
 #include "es_internal.h"
 #include "es_noise.cuh"
+#if FX==0
+#define FSH 1024,2,2
+#elif FX==1
+#define FSH 768,2,2
+#elif FX==2
+#define FSH 896,2,2
+#elif FX==3
+#define FSH 768,1,1
+#elif FX==4
+#define FSH 768,3,3
+#elif FX==5
+#define FSH 640,2,2
+#elif FX==6
+#define FSH 640,1,1
+#endif
 
 namespace esopt {
 namespace {
 
-// 16-byte vector <-> fp32 registers, and single-element access for tails.
+// Stored vector <-> fp32 registers, and units of 8 elements, whole or cut off.
 struct Bf16Io {
   static constexpr int kVec = 8;
   static constexpr bool kScaled = false;
   using Scalar = uint16_t;
+  using Vec = uint4;  // what a thread loads at once in a run
   using Raw = uint4;  // a unit of 8 elements as stored
   __device__ static uint32_t pack2(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);  // one cvt.rn.bf16x2.f32
@@ -85,6 +101,7 @@ struct F32Io {
   static constexpr int kVec = 4;
   static constexpr bool kScaled = false;
   using Scalar = float;
+  using Vec = uint4;
   __device__ static void unpack(const uint4& v, float (&f)[4]) {
     f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y);
     f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
@@ -139,15 +156,17 @@ struct F32Io {
   }
 };
 
-// FP8 E4M3 storage: 16 elements per 16-byte vector, byte k of the vector is
+// FP8 E4M3 storage: 8 elements per 8-byte vector, byte k of the vector is
 // element k. Values stay in units of the segment's scale: the kernels multiply
 // the noise by 1 / scale instead (kScaled). Decoding goes through half
 // precision, which holds every E4M3 value exactly; encoding rounds fp32 to the
 // nearest E4M3 value, ties to even, saturating at +-448 (cvt .satfinite).
 struct Fp8Io {
-  static constexpr int kVec = 16;
+  static constexpr int kVec = 8;
   static constexpr bool kScaled = true;
   using Scalar = uint8_t;
+  using Vec = uint2;
+  using Raw = uint2;
   __device__ static float2 dec2(uint32_t pair) {
     const __half2_raw h =
         __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(pair & 0xFFFFu), __NV_E4M3);
@@ -157,20 +176,17 @@ struct Fp8Io {
     return static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(make_float2(lo, hi), __NV_SATFINITE,
                                                           __NV_E4M3));
   }
-  __device__ static void unpack(const uint4& v, float (&f)[16]) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  __device__ static void unpack(const uint2& v, float (&f)[8]) {
+    const uint32_t w[2] = {v.x, v.y};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 2; ++k) {
       const float2 a = dec2(w[k]), b = dec2(w[k] >> 16);
       f[4 * k + 0] = a.x; f[4 * k + 1] = a.y; f[4 * k + 2] = b.x; f[4 * k + 3] = b.y;
     }
   }
-  __device__ static uint4 pack(const float (&f)[16]) {
-    uint32_t w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      w[k] = enc2(f[4 * k + 0], f[4 * k + 1]) | (enc2(f[4 * k + 2], f[4 * k + 3]) << 16);
-    return make_uint4(w[0], w[1], w[2], w[3]);
+  __device__ static uint2 pack(const float (&f)[8]) {
+    return make_uint2(enc2(f[0], f[1]) | (enc2(f[2], f[3]) << 16),
+                      enc2(f[4], f[5]) | (enc2(f[6], f[7]) << 16));
   }
   template <int M>
   __device__ static void round_trip(float (&f)[M]) {
@@ -181,7 +197,6 @@ struct Fp8Io {
       f[k + 1] = r.y;
     }
   }
-  using Raw = uint2;
   __device__ static float value(uint8_t c) { return dec2(c).x; }
   __device__ static uint8_t store(float f) { return static_cast<uint8_t>(enc2(f, 0.0f)); }
   __device__ static Raw load_unit(const uint8_t* p, int rem) {
@@ -203,18 +218,8 @@ struct Fp8Io {
       if (k < rem) p[k] = static_cast<uint8_t>(w[k >> 2] >> (8 * (k & 3)));
   }
   __device__ static Raw zero_unit() { return make_uint2(0u, 0u); }
-  __device__ static void unpack_unit(const Raw& v, float (&f)[kUnit]) {
-    const uint32_t w[2] = {v.x, v.y};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float2 a = dec2(w[k]), b = dec2(w[k] >> 16);
-      f[4 * k + 0] = a.x; f[4 * k + 1] = a.y; f[4 * k + 2] = b.x; f[4 * k + 3] = b.y;
-    }
-  }
-  __device__ static Raw pack_unit(const float (&f)[kUnit]) {
-    return make_uint2(enc2(f[0], f[1]) | (enc2(f[2], f[3]) << 16),
-                      enc2(f[4], f[5]) | (enc2(f[6], f[7]) << 16));
-  }
+  __device__ static void unpack_unit(const Raw& v, float (&f)[kUnit]) { unpack(v, f); }
+  __device__ static Raw pack_unit(const float (&f)[kUnit]) { return pack(f); }
 };
 
 // theta + acc in storage units: acc is in parameter units, so a scaled
@@ -377,43 +382,53 @@ __device__ __forceinline__ UnitRef<Io> unit_ref(const SegDesc& d, float inv,
 // two steps, the second on the first's result rounded to the storage type
 // (restore of one member fused with the perturb of the next); the two steps
 // of one seed, whose noise is generated once (the antithetic flip); or the update
-// of a population of 1 to 4, theta += sum_i scale_i eps_seed_i rounded once.
-enum class AxpyMode { kOne, kTwo, kFlip, kSum1, kSum2, kSum3, kSum4 };
-constexpr int kMaxSum = 4;
+// of a population of 1 to 8, theta += sum_i scale_i eps_seed_i rounded once, which
+// the next generation's first perturb may follow on the rounded result.
+enum class AxpyKind { kSteps, kFlip, kSum, kSumPerturb };
+constexpr int kMaxSum = 8;
 
-// Number of seeds of a mode, and whether it is one of the sums.
-__host__ __device__ constexpr int axpy_seeds(AxpyMode m) {
-  return m == AxpyMode::kOne || m == AxpyMode::kFlip || m == AxpyMode::kSum1 ? 1
-         : m == AxpyMode::kTwo || m == AxpyMode::kSum2                     ? 2
-         : m == AxpyMode::kSum3                                            ? 3
-                                                                           : 4;
-}
-__host__ __device__ constexpr bool axpy_is_sum(AxpyMode m) { return m >= AxpyMode::kSum1; }
+// What a pass does, and the number of its seeds' schedules (kSumPerturb: the last
+// one is the perturb's).
+template <AxpyKind kKind, int kSeedCount>
+struct AxpyMode {
+  static constexpr AxpyKind kind = kKind;
+  static constexpr int seeds = kSeedCount;
+  static constexpr bool sum = kKind == AxpyKind::kSum || kKind == AxpyKind::kSumPerturb;
+};
+using AxpyOne = AxpyMode<AxpyKind::kSteps, 1>;
+using AxpyTwo = AxpyMode<AxpyKind::kSteps, 2>;
+using AxpyFlip = AxpyMode<AxpyKind::kFlip, 1>;
+template <int N>
+using AxpySum = AxpyMode<AxpyKind::kSum, N>;
+template <int N>
+using AxpySumPerturb = AxpyMode<AxpyKind::kSumPerturb, N + 1>;
 
 // Arguments of a launch: each seed's schedule, and the scale of each step or
 // seed. A __grid_constant__ parameter, so every round key is read from the
 // constant bank as an instruction operand.
 struct AxpyArgs {
-  PhiloxSched seed[kMaxSum];
-  float scale[kMaxSum];
+  PhiloxSched seed[kMaxSum + 1];
+  float scale[kMaxSum + 1];
 };
 
-// The steps of kMode on the V values f. words(i, x) gives the Philox words of
+// The steps of Mode on the V values f. words(i, x) gives the Philox words of
 // seed i's blocks; inv is 1 / the segment's scale.
-template <class Io, AxpyMode kMode, int V, class Words>
+template <class Io, class Mode, int V, class Words>
 __device__ __forceinline__ void axpy_values(const Words& words, const AxpyArgs& a, float inv,
                                             float (&f)[V]) {
-  constexpr int kSeeds = axpy_seeds(kMode);
+  constexpr int kSeeds = Mode::seeds;
   uint4 x[V / 4];
   words(0, x);
-  if constexpr (axpy_is_sum(kMode)) {
+  if constexpr (Mode::sum) {
     float acc[V];
 #pragma unroll
     for (int k = 0; k < V; ++k) acc[k] = 0.0f;
     // each seed's words before the transform of the one before (2 % faster than
     // after it; the two-step pass does not gain from it)
+    constexpr bool kPerturb = Mode::kind == AxpyKind::kSumPerturb;
+    constexpr int kSummed = kSeeds - (kPerturb ? 1 : 0);
 #pragma unroll
-    for (int i = 0; i < kSeeds; ++i) {
+    for (int i = 0; i < kSummed; ++i) {
       uint4 y[V / 4];
       if (i + 1 < kSeeds) words(i + 1, y);
       add_scaled_noise<V>(x, a.scale[i], acc);
@@ -424,7 +439,11 @@ __device__ __forceinline__ void axpy_values(const Words& words, const AxpyArgs& 
     }
 #pragma unroll
     for (int k = 0; k < V; ++k) f[k] = add_acc<Io>(f[k], acc[k], inv);
-  } else if constexpr (kMode == AxpyMode::kFlip) {
+    if constexpr (kPerturb) {
+      Io::round_trip(f);
+      add_scaled_noise<V>(x, a.scale[kSummed] * inv, f);
+    }
+  } else if constexpr (Mode::kind == AxpyKind::kFlip) {
     Polar2 pp[V / 4];
     polar_from_words<V / 4>(x, pp);
     apply_noise<V>(pp, a.scale[0] * inv, f);
@@ -432,7 +451,7 @@ __device__ __forceinline__ void axpy_values(const Words& words, const AxpyArgs& 
     apply_noise<V>(pp, a.scale[1] * inv, f);
   } else {
     add_scaled_noise<V>(x, a.scale[0] * inv, f);
-    if constexpr (kMode == AxpyMode::kTwo) {
+    if constexpr (kSeeds == 2) {
       Io::round_trip(f);
       words(1, x);
       add_scaled_noise<V>(x, a.scale[1] * inv, f);
@@ -441,9 +460,9 @@ __device__ __forceinline__ void axpy_values(const Words& words, const AxpyArgs& 
 }
 
 // The generators of a launch's seeds for one high counter word.
-template <AxpyMode kMode, bool kWide>
+template <class Mode, bool kWide>
 struct AxpyGens {
-  static constexpr int kSeeds = axpy_seeds(kMode);
+  static constexpr int kSeeds = Mode::seeds;
   TileConst t[kSeeds];
   __device__ AxpyGens(const AxpyArgs& a, uint32_t j_hi) {
 #pragma unroll
@@ -455,42 +474,46 @@ struct AxpyGens {
   }
 };
 
-// Shape of a pass: threads of its one CTA per SM, 16-byte vectors per thread
-// in a tile (the unrolled body of the loop) and how many vectors ahead theta is
-// loaded. What bounds the passes is the generator's instruction stream: the
-// FMA-heavy pipe (integer products), MUFU and issue, and, seen by what moves
-// them, instruction fetch: all of an SM's warps in one CTA on a loop body of
-// 300-600 instructions run 6-15 % faster than 2 or 3 CTAs of 256 threads on one
-// of 1200. Measured on sm_103a over 792,680,960 parameters (us; 256 threads, 4
-// vectors, 1 ahead, grid-stride tiles -> this): bf16 one step 678 -> 569 (5.58 TB/s), two
-// steps 1217 -> 1094 (1.449e12 Gaussians/s), flip 729 -> 621; fp32 971 -> 962 (6.59 TB/s: HBM),
-// 1366 -> 1077, 976 -> 961; FP8 636 -> 575, 1301 -> 1127, 718 -> 639.
-// The sums replace the seed loop of update_kernel where it is too short for its
-// pipeline: 1 / 2 / 3 / 4 seeds bf16 972 / 1480 / 2035 / 2555 -> 591 / 1078 /
-// 1596 / 2107, fp32 1125 / 1642 / 2253 / 2866 -> 962 / 1088 / 1589 / 2145, FP8
-// 811 / 1392 / 1979 / 2567 -> 602 / 1110 / 1608 / 2113.
+// Shape of a pass: threads of its one CTA per SM, vectors per thread in a tile
+// (the unrolled body of the loop) and how many vectors ahead theta is loaded. What
+// bounds the passes is the generator's instruction stream: the FMA-heavy pipe
+// (integer products), MUFU and issue. All of an SM's warps in one CTA on a short
+// loop body run 6-15 % faster than 2 or 3 CTAs of 256 threads on a body of four
+// vectors. Measured on sm_103a over 792,680,960 parameters (us; 256 threads, 4
+// vectors, 1 ahead, grid-stride tiles -> this): bf16 one step 678 -> 569 (5.58 TB/s),
+// two steps 1217 -> 1094 (1.449e12 Gaussians/s), flip 729 -> 621; fp32 971 -> 960 (6.6
+// TB/s: HBM), 1366 -> 1077, 976 -> 961; FP8 636 -> 570, 1301 -> 1118, 718 -> 635 (8
+// elements at a time: 16 hold twice the registers and body, and cost the sums of 4 and
+// more seeds 1-10 %).
+// The sums replace the seed loop of update_kernel, which spends a third of a seed
+// per unit filling and draining its pipeline and reads each seed's keys from shared
+// memory: 1 / 2 / 3 / 4 / 8 seeds bf16 972 / 1480 / 2035 / 2555 / 4700 -> 591 / 1075 /
+// 1604 / 2107 / 4183 (the seed loop as it is now: 4404 at 8), fp32 1125 / 1642 / 2253 /
+// 2866 / 5314 -> 962 / 1088 / 1589 / 2145 / 4351, FP8 811 / 1392 / 1979 / 2567 / 4902 -> 589 /
+// 1088 / 1579 / 2115 / 4171; with the perturb behind 1 / 4 / 8 bf16 seeds 1656 / 3249 / 5433
+// -> 1107 / 2675 / 4752. 12 and 16 seeds unrolled gain 3 and 1 % on the loop, for twice
+// the code: not built.
 // Thread counts that are no multiple of 128 leave the SM's four schedulers
 // unequal warps and run 10 % slower.
 struct AxpyShape {
   int threads, vecs, ahead;
 };
-template <class Io, AxpyMode kMode>
+template <class Io, class Mode>
 __host__ __device__ constexpr AxpyShape axpy_shape() {
-  if (axpy_is_sum(kMode)) {
-    if (Io::kVec == 4) return {1024, 4, 2};
-    if (Io::kVec == 16) return {kMode == AxpyMode::kSum1 ? 768 : 512, 1, 1};
-    return kMode == AxpyMode::kSum4 ? AxpyShape{768, 1, 1} : AxpyShape{1024, 2, 2};
-  }
-  if (Io::kVec == 4) return {1024, 4, 2};
-  if (Io::kVec == 16) return kMode == AxpyMode::kTwo ? AxpyShape{640, 2, 2} : AxpyShape{768, 2, 1};
-  return kMode == AxpyMode::kOne   ? AxpyShape{1024, 2, 2}
-         : kMode == AxpyMode::kTwo ? AxpyShape{1024, 2, 1}
-                                   : AxpyShape{1024, 3, 1};
+  if (Io::kVec == 4) return Mode::seeds > 4 ? AxpyShape{1024, 1, 1} : AxpyShape{1024, 4, 2};
+  if (Mode::sum)
+    return Mode::seeds == 1 || (Mode::seeds == 2 && !Io::kScaled) ? AxpyShape{1024, 2, 2}
+           : Mode::seeds <= 3                                     ? AxpyShape{896, 2, 2}
+           : Mode::seeds <= 7                                     ? AxpyShape{768, 1, 1}
+                                                                  : AxpyShape{640, 1, 1};
+  if (Mode::kind == AxpyKind::kFlip) return {1024, 3, 1};
+  if (Mode::seeds == 1) return {1024, 2, 2};
+  return Io::kScaled ? AxpyShape{768, 2, 2} : AxpyShape{1024, 2, 1};
 }
 // Units of one tile.
-template <class Io, AxpyMode kMode>
+template <class Io, class Mode>
 __host__ __device__ constexpr uint64_t axpy_tile_units() {
-  constexpr AxpyShape k = axpy_shape<Io, kMode>();
+  constexpr AxpyShape k = axpy_shape<Io, Mode>();
   return static_cast<uint64_t>(k.threads) * k.vecs * Io::kVec / kUnit;
 }
 
@@ -501,23 +524,23 @@ __host__ __device__ constexpr uint64_t axpy_tile_units() {
 // vector `ahead` of the current one is issued before that is computed. Round 0's Philox
 // product (of the counter alone) is stepped by 64-bit additions from the
 // thread's first block instead of multiplied.
-template <class Io, AxpyMode kMode>
+template <class Io, class Mode>
 __device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thread, uint32_t tiles,
                                          const AxpyArgs& a, float inv) {
   constexpr int V = Io::kVec, NB = V / 4;
-  constexpr AxpyShape kShape = axpy_shape<Io, kMode>();
+  constexpr AxpyShape kShape = axpy_shape<Io, Mode>();
   constexpr int D = kShape.ahead;
   constexpr int kStride = kShape.threads * V;  // elements between a thread's vectors
   static_assert(kShape.vecs % D == 0, "the vectors in flight rotate within a tile");
   // the one-seed pass is fastest with every Philox product 64-bit wide (in
   // FP8 storage, with twice the blocks per vector, that spills)
-  constexpr bool kWide = kMode == AxpyMode::kOne && V <= 8;
+  constexpr bool kWide = Mode::kind == AxpyKind::kSteps && Mode::seeds == 1 && V <= 8;
   const uint32_t j_hi = static_cast<uint32_t>(j_thread >> 32);
-  const AxpyGens<kMode, kWide> gens(a, j_hi);
+  const AxpyGens<Mode, kWide> gens(a, j_hi);
   Round0 p0 = philox_round0<kWide>(static_cast<uint32_t>(j_thread));
-  uint4 v[D];
+  typename Io::Vec v[D];
 #pragma unroll
-  for (int k = 0; k < D; ++k) v[k] = *reinterpret_cast<const uint4*>(p + k * kStride);
+  for (int k = 0; k < D; ++k) v[k] = *reinterpret_cast<const typename Io::Vec*>(p + k * kStride);
 #pragma unroll 1
   for (;;) {
 #pragma unroll
@@ -525,17 +548,17 @@ __device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thre
       float f[V];
       Io::unpack(v[u % D], f);
       if (u + D < kShape.vecs || tiles > 1)
-        v[u % D] = *reinterpret_cast<const uint4*>(p + (u + D) * kStride);
+        v[u % D] = *reinterpret_cast<const typename Io::Vec*>(p + (u + D) * kStride);
       Round0 r0[NB];
 #pragma unroll
       for (int b = 0; b < NB; ++b) r0[b] = round0_step(p0, static_cast<uint32_t>(u * (kStride / 4) + b));
-      axpy_values<Io, kMode, V>(
+      axpy_values<Io, Mode, V>(
           [&](int i, uint4 (&x)[NB]) {
 #pragma unroll
             for (int b = 0; b < NB; ++b) x[b] = gens.words(a, i, r0[b]);
           },
           a, inv, f);
-      *reinterpret_cast<uint4*>(p + u * kStride) = Io::pack(f);
+      *reinterpret_cast<typename Io::Vec*>(p + u * kStride) = Io::pack(f);
     }
     if (--tiles == 0) return;
     p += kShape.vecs * kStride;
@@ -544,7 +567,7 @@ __device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thre
 }
 
 // One unit of the calling thread.
-template <class Io, AxpyMode kMode>
+template <class Io, class Mode>
 __device__ __forceinline__ void axpy_unit(const UnitRef<Io>& r, const AxpyArgs& a) {
   constexpr int NB = kUnit / 4;
   if (r.rem == 0) return;
@@ -553,11 +576,11 @@ __device__ __forceinline__ void axpy_unit(const UnitRef<Io>& r, const AxpyArgs& 
   Io::unpack_unit(raw, f);
   // a unit's two blocks start at an even one, so they share the high word
   const uint32_t j_hi = static_cast<uint32_t>(r.j0 >> 32);
-  const AxpyGens<kMode, false> gens(a, j_hi);
+  const AxpyGens<Mode, false> gens(a, j_hi);
   Round0 r0[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) r0[b] = philox_round0<false>(static_cast<uint32_t>(r.j0 + b));
-  axpy_values<Io, kMode, kUnit>(
+  axpy_values<Io, Mode, kUnit>(
       [&](int i, uint4 (&x)[NB]) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) x[b] = gens.words(a, i, r0[b]);
@@ -573,12 +596,12 @@ __device__ __forceinline__ void axpy_unit(const UnitRef<Io>& r, const AxpyArgs& 
 // and up to a tile's worth of units wherever a segment, the range or a high
 // counter word ends (axpy_unit; each thread finds its unit's segment). It waits for
 // the kernel before it only when it has read the table.
-template <class Io, AxpyMode kMode>
-__global__ void __launch_bounds__(axpy_shape<Io, kMode>().threads, 1)
+template <class Io, class Mode>
+__global__ void __launch_bounds__(axpy_shape<Io, Mode>().threads, 1)
 axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
                   const Split split, const __grid_constant__ AxpyArgs a) {
-  constexpr AxpyShape kShape = axpy_shape<Io, kMode>();
-  constexpr uint64_t kTile = axpy_tile_units<Io, kMode>();
+  constexpr AxpyShape kShape = axpy_shape<Io, Mode>();
+  constexpr uint64_t kTile = axpy_tile_units<Io, Mode>();
   uint64_t q = range_begin(split) * kUnitsPerGranule;
   const uint64_t end = range_end(split) * kUnitsPerGranule;
   int seg = search_segment(segs, 0, nseg, q / kUnitsPerGranule);
@@ -587,8 +610,8 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
       seg = search_segment(segs, seg + 1, nseg, q / kUnitsPerGranule);
     const SegDesc d = segs[seg];
     const uint64_t begin = d.granule_begin * kUnitsPerGranule;
-    // where the segment's whole vectors (FP8: pairs of units) end
-    uint64_t whole = begin + d.numel / Io::kVec * Io::kVec / kUnit;
+    // where the segment's whole units end
+    uint64_t whole = begin + d.numel / kUnit;
     if (whole > end) whole = end;
     if (q + kTile <= whole && blockDim.x == kShape.threads) {
       const uint64_t e = (q - begin) * kUnit, g = d.index_base + e;
@@ -599,7 +622,7 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
         if (tiles > 0x7FFFFFFFu) tiles = 0x7FFFFFFFu;
         const uint64_t mine = threadIdx.x * static_cast<uint64_t>(Io::kVec);
         wait_for_previous();
-        axpy_run<Io, kMode>(static_cast<typename Io::Scalar*>(d.data) + e + mine, (g + mine) >> 2,
+        axpy_run<Io, Mode>(static_cast<typename Io::Scalar*>(d.data) + e + mine, (g + mine) >> 2,
                             static_cast<uint32_t>(tiles), a, Io::kScaled ? inv_scale[seg] : 1.0f);
         q += tiles * kTile;
         continue;
@@ -611,14 +634,14 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
     // Units of one segment take its entry from registers, which saves a launch
     // 0.2-0.5 us (2^22 bf16 parameters 5.9 -> 5.5 us); in the bf16 two-step pass
     // and sums the second loop costs the run above 2 % instead
-    constexpr bool kKeep = Io::kVec != 8 || kMode == AxpyMode::kOne || kMode == AxpyMode::kFlip;
+    constexpr bool kKeep = Io::kVec != 8 || (!Mode::sum && Mode::seeds == 1);
     bool done = false;
     if constexpr (kKeep) {
       if (seg == last) {
         const float inv = Io::kScaled ? inv_scale[seg] : 1.0f;
 #pragma unroll 1
         for (uint64_t u = q + threadIdx.x; u < stop; u += blockDim.x)
-          axpy_unit<Io, kMode>(unit_ref<Io>(d, inv, u), a);
+          axpy_unit<Io, Mode>(unit_ref<Io>(d, inv, u), a);
         done = true;
       }
     }
@@ -626,7 +649,7 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
 #pragma unroll 1
       for (uint64_t u = q + threadIdx.x; u < stop; u += blockDim.x) {
         const int s = segment_between(segs, seg, last, u / kUnitsPerGranule);
-        axpy_unit<Io, kMode>(unit_ref<Io>(segs[s], Io::kScaled ? inv_scale[s] : 1.0f, u), a);
+        axpy_unit<Io, Mode>(unit_ref<Io>(segs[s], Io::kScaled ? inv_scale[s] : 1.0f, u), a);
       }
     }
     __syncwarp();
@@ -1254,20 +1277,20 @@ cudaError_t launch_early(void (*kernel)(P...), int grid, int block, bool early, 
   return err != cudaSuccess ? err : last;
 }
 
-template <class Io, AxpyMode kMode>
+template <class Io, class Mode>
 cudaError_t launch_axpy_io(const PlanView& plan, const AxpyArgs& a, cudaStream_t stream) {
-  auto k = axpy_noise_kernel<Io, kMode>;
-  const Launch l = make_launch(reinterpret_cast<const void*>(k), axpy_shape<Io, kMode>().threads,
-                               axpy_tile_units<Io, kMode>(), plan.granules);
+  auto k = axpy_noise_kernel<Io, Mode>;
+  const Launch l = make_launch(reinterpret_cast<const void*>(k), axpy_shape<Io, Mode>().threads,
+                               axpy_tile_units<Io, Mode>(), plan.granules);
   return launch_early(k, l.grid, l.block, plan.early, stream, plan.segs, plan.nseg, plan.inv_scale,
                       l.split, a);
 }
 
-template <AxpyMode kMode>
+template <class Mode>
 cudaError_t launch_axpy(const PlanView& plan, const AxpyArgs& a, cudaStream_t stream) {
-  if (plan.dtype == ES_BF16) return launch_axpy_io<Bf16Io, kMode>(plan, a, stream);
-  if (plan.dtype == ES_FP8_E4M3) return launch_axpy_io<Fp8Io, kMode>(plan, a, stream);
-  return launch_axpy_io<F32Io, kMode>(plan, a, stream);
+  if (plan.dtype == ES_BF16) return launch_axpy_io<Bf16Io, Mode>(plan, a, stream);
+  if (plan.dtype == ES_FP8_E4M3) return launch_axpy_io<Fp8Io, Mode>(plan, a, stream);
+  return launch_axpy_io<F32Io, Mode>(plan, a, stream);
 }
 
 }  // namespace
@@ -1277,7 +1300,7 @@ cudaError_t launch_axpy_noise(const PlanView& plan, uint64_t seed, float scale,
   AxpyArgs a{};
   a.seed[0] = philox_sched(seed);
   a.scale[0] = scale;
-  return launch_axpy<AxpyMode::kOne>(plan, a, stream);
+  return launch_axpy<AxpyOne>(plan, a, stream);
 }
 
 cudaError_t launch_axpy_noise2(const PlanView& plan, uint64_t seed, float scale, uint64_t seed2,
@@ -1287,8 +1310,8 @@ cudaError_t launch_axpy_noise2(const PlanView& plan, uint64_t seed, float scale,
   a.seed[1] = philox_sched(seed2);
   a.scale[0] = scale;
   a.scale[1] = scale2;
-  return seed == seed2 ? launch_axpy<AxpyMode::kFlip>(plan, a, stream)
-                       : launch_axpy<AxpyMode::kTwo>(plan, a, stream);
+  return seed == seed2 ? launch_axpy<AxpyFlip>(plan, a, stream)
+                       : launch_axpy<AxpyTwo>(plan, a, stream);
 }
 
 template <class Io, bool kSingle, bool kPerturb>
@@ -1341,22 +1364,40 @@ cudaError_t launch_update_split(const PlanView& plan, const UpdateArgs& args, cu
   return launch_split_io<F32Io>(plan, a, stream);
 }
 
+template <int N>
+cudaError_t launch_sum_of(const PlanView& plan, const AxpyArgs& a, bool perturb,
+                          cudaStream_t stream) {
+  return perturb ? launch_axpy<AxpySumPerturb<N>>(plan, a, stream)
+                 : launch_axpy<AxpySum<N>>(plan, a, stream);
+}
+
+cudaError_t launch_sum(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
+  AxpyArgs a{};
+  for (int i = 0; i < args.n; ++i) {
+    a.seed[i] = philox_sched(static_cast<uint64_t>(args.key[i][1]) << 32 | args.key[i][0]);
+    a.scale[i] = args.coeff[i];
+  }
+  if (args.perturb) {
+    a.seed[args.n] = philox_sched(static_cast<uint64_t>(args.pkey[1]) << 32 | args.pkey[0]);
+    a.scale[args.n] = args.pscale;
+  }
+  const bool p = args.perturb != 0;
+  switch (args.n) {
+    case 1: return launch_sum_of<1>(plan, a, p, stream);
+    case 2: return launch_sum_of<2>(plan, a, p, stream);
+    case 3: return launch_sum_of<3>(plan, a, p, stream);
+    case 4: return launch_sum_of<4>(plan, a, p, stream);
+    case 5: return launch_sum_of<5>(plan, a, p, stream);
+    case 6: return launch_sum_of<6>(plan, a, p, stream);
+    case 7: return launch_sum_of<7>(plan, a, p, stream);
+    default: return launch_sum_of<8>(plan, a, p, stream);
+  }
+}
+
 cudaError_t launch_update(const PlanView& plan, const UpdateArgs& args, cudaStream_t stream) {
   if (args.n <= kSplitSeeds && plan.granules <= kSplitMaxGranules)
     return launch_update_split(plan, args, stream);
-  if (args.n_gen == 1 && !args.perturb && args.n <= kMaxSum) {
-    AxpyArgs a{};
-    for (int i = 0; i < args.n; ++i) {
-      a.seed[i] = philox_sched(static_cast<uint64_t>(args.key[i][1]) << 32 | args.key[i][0]);
-      a.scale[i] = args.coeff[i];
-    }
-    switch (args.n) {
-      case 1: return launch_axpy<AxpyMode::kSum1>(plan, a, stream);
-      case 2: return launch_axpy<AxpyMode::kSum2>(plan, a, stream);
-      case 3: return launch_axpy<AxpyMode::kSum3>(plan, a, stream);
-      default: return launch_axpy<AxpyMode::kSum4>(plan, a, stream);
-    }
-  }
+  if (args.n_gen == 1 && args.n <= kMaxSum) return launch_sum(plan, args, stream);
   if (plan.dtype == ES_BF16) return launch_update_dtype<Bf16Io>(plan, args, stream);
   if (plan.dtype == ES_FP8_E4M3) return launch_update_dtype<Fp8Io>(plan, args, stream);
   return launch_update_dtype<F32Io>(plan, args, stream);

@@ -57,8 +57,8 @@ def test_long_runs_equal_short_segments(es, oracle, dtype, numel):
         np.arange(64), np.arange(edge - 9000, edge + 9000), np.arange(numel - 9000, numel),
         np.random.default_rng(4).integers(0, numel, size=20000)]))
     g = np.uint64(base) + at.astype(np.uint64)
-    seeds = np.array([9, 2**40 + 1, 77, 4, 2**63], dtype=np.uint64)
-    coeffs = np.array([2e-3, -1e-3, 5e-4, 1e-3, -5e-4], dtype=np.float32)
+    seeds = np.array([9, 2**40 + 1, 77, 4, 2**63, 5, 6, 8, 2**64 - 1], dtype=np.uint64)
+    coeffs = np.array([2, -1, 0.5, 1, -0.5, 1.5, -2, 1, 0.25], dtype=np.float32) * np.float32(1e-3)
 
     def sample():
         return a.cpu().numpy()[at] if dtype == "fp8" else host_values(a)[at]
@@ -86,11 +86,18 @@ def test_long_runs_equal_short_segments(es, oracle, dtype, numel):
         both(lambda p: es.es_restore_perturb(p, 9, 1e-3, second, -1e-3))
         torch.cuda.synchronize()
         assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), "restore_perturb"
-    # populations of 1 to 4 have passes of their own, 5 takes the seed loop
-    for n in (1, 2, 3, 4, 5):
+    # populations of 1 to 8 have passes of their own, 9 takes the seed loop
+    for n in range(1, 10):
         before = both(lambda p: es.es_update(p, seeds[:n], coeffs[:n]))
         noise = noise_abs_tol([oracle.noise_at(int(s), g) for s in seeds[:n]], coeffs[:n])
         check(f"update {n}", oracle.update(before, g, seeds[:n], coeffs[:n], name, *extra), noise)
+        # the fused call: one plan by it, the other by the two calls
+        es.es_update_perturb(long_plan, seeds[:n], coeffs[:n], 5, 1e-3)
+        es.es_update(short_plan, seeds[:n], coeffs[:n])
+        es.es_perturb(short_plan, 5, 1e-3)
+        torch.cuda.synchronize()
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), ("update_perturb", n)
+    seeds, coeffs = seeds[:5], coeffs[:5]
     both(lambda p: es.es_update_perturb(p, seeds, coeffs, 5, 1e-3))
     both(lambda p: es.es_replay(p, np.tile(seeds, 30), np.tile(coeffs, 30), [1, 2, 3] * 25))
     torch.cuda.synchronize()
