@@ -351,25 +351,27 @@ es_status_t es_fold_antithetic(const double* rhat_pos, const double* rhat_neg,
  * current device, 16-byte aligned data, index bases multiples of 8, no
  * overlap) and are validated on every call.
  *
- * Instead of a plan's table, the segment table is copied (cudaMemcpyAsync on
- * `stream`) into one static device array of ES_STATIC_MAX_SEGMENTS + 1
- * descriptors (about 32 KB), which every device that loads the library holds
- * until the process exits. The entry point calls no cudaMalloc, cudaFree or
- * other allocating routine, and uses about 36 KB of host stack.
+ * Instead of a plan's table, a table of up to 64 segments travels with the launch
+ * itself; a longer one is copied (cudaMemcpyAsync on `stream`) into one static
+ * device array of ES_STATIC_MAX_SEGMENTS + 1 descriptors (about 32 KB), which every
+ * device that loads the library holds until the process exits. The entry point
+ * calls no cudaMalloc, cudaFree or other allocating routine, and uses about 38 KB
+ * of host stack.
  *   - More than ES_STATIC_MAX_SEGMENTS segments: ES_ERR_INVALID_ARG, nothing
  *     is launched.
- *   - All calls share the one array and each call rewrites it whole (nothing
- *     in it needs to start at zero); it keeps the last call's table. Calls
- *     that overlap on the GPU (on different streams, or from several host
- *     threads without ordering) race on that array and must not be issued.
- *   - The first call on each device looks up the array's device address
+ *   - Calls of more than 64 segments share the one array and each rewrites it
+ *     whole (nothing in it needs to start at zero); it keeps the last such call's
+ *     table. Such calls that overlap on the GPU (on different streams, or from
+ *     several host threads without ordering) race on that array and must not be
+ *     issued.
+ *   - The first such call on each device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current and keeps it for that
  *     device's context (after a device reset the next call looks it up
  *     again); make that first call before any stream capture.
  *   - A call on a stream that is being captured is refused with
- *     ES_ERR_INVALID_ARG before anything is copied or launched: the table is
- *     copied from the call's own stack, which a recorded copy would read again
- *     long after the call has returned.
+ *     ES_ERR_INVALID_ARG before anything is copied or launched, whatever its
+ *     number of segments: a longer table is copied from the call's own stack, which
+ *     a recorded copy would read again long after the call has returned.
  * Errors: ES_ERR_INVALID_ARG, ES_ERR_ALIGNMENT, ES_ERR_OVERLAP,
  * ES_ERR_NONFINITE, ES_ERR_CUDA.
  */

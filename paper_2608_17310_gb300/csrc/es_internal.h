@@ -34,6 +34,12 @@ struct SegDesc {
 };
 static_assert(sizeof(SegDesc) == 32, "SegDesc layout");
 
+// A segment table small enough to travel as a launch parameter (2 KB).
+constexpr int kTableSegments = 64;
+struct SegTable {
+  SegDesc entry[kTableSegments + 1];
+};
+
 // Largest number of generations one fused update launch applies.
 constexpr int kMaxGenerations = 256;
 
@@ -69,6 +75,10 @@ struct PlanView {
 // Kernel launchers (es_kernels.cu). Each returns the launch's cudaError_t.
 cudaError_t launch_axpy_noise(const PlanView& plan, uint64_t seed, float scale,
                               cudaStream_t stream);
+// The same on bf16 or fp32 segments without a plan: nseg <= kTableSegments entries
+// and the sentinel.
+cudaError_t launch_axpy_table(const SegTable& table, int nseg, es_dtype_t dtype, uint64_t seed,
+                              float scale, cudaStream_t stream);
 cudaError_t launch_axpy_noise2(const PlanView& plan, uint64_t seed, float scale, uint64_t seed2,
                                float scale2, cudaStream_t stream);  // seed2 may equal seed
 cudaError_t launch_update(const PlanView& plan, const UpdateArgs& args,

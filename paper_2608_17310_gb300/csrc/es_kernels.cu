@@ -597,9 +597,9 @@ __device__ __forceinline__ void axpy_unit(const UnitRef<Io>& r, const AxpyArgs& 
 // counter word ends (axpy_unit; each thread finds its unit's segment). It waits for
 // the kernel before it only when it has read the table.
 template <class Io, class Mode>
-__global__ void __launch_bounds__(axpy_shape<Io, Mode>().threads, 1)
-axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
-                  const Split split, const __grid_constant__ AxpyArgs a) {
+__device__ __forceinline__ void axpy_pass(const SegDesc* __restrict__ segs, int nseg,
+                                          const float* __restrict__ inv_scale, const Split& split,
+                                          const AxpyArgs& a) {
   constexpr AxpyShape kShape = axpy_shape<Io, Mode>();
   constexpr uint64_t kTile = axpy_tile_units<Io, Mode>();
   uint64_t q = range_begin(split) * kUnitsPerGranule;
@@ -657,6 +657,22 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
     seg = last;
   }
   let_next_start();
+}
+
+template <class Io, class Mode>
+__global__ void __launch_bounds__(axpy_shape<Io, Mode>().threads, 1)
+axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
+                  const Split split, const __grid_constant__ AxpyArgs a) {
+  axpy_pass<Io, Mode>(segs, nseg, inv_scale, split, a);
+}
+
+// The same with the segment table in the launch's parameters, for a caller without a
+// plan: no copy goes ahead of the kernel in its stream.
+template <class Io, class Mode>
+__global__ void __launch_bounds__(axpy_shape<Io, Mode>().threads, 1)
+axpy_table_kernel(const __grid_constant__ SegTable table, int nseg, const Split split,
+                  const __grid_constant__ AxpyArgs a) {
+  axpy_pass<Io, Mode>(table.entry, nseg, nullptr, split, a);
 }
 
 // Seeds of an update launch are staged in shared memory kSchedRows at a time,
@@ -1301,6 +1317,24 @@ cudaError_t launch_axpy_noise(const PlanView& plan, uint64_t seed, float scale,
   a.seed[0] = philox_sched(seed);
   a.scale[0] = scale;
   return launch_axpy<AxpyOne>(plan, a, stream);
+}
+
+template <class Io>
+cudaError_t launch_table_io(const SegTable& table, int nseg, const AxpyArgs& a,
+                            cudaStream_t stream) {
+  auto k = axpy_table_kernel<Io, AxpyOne>;
+  const Launch l = make_launch(reinterpret_cast<const void*>(k), axpy_shape<Io, AxpyOne>().threads,
+                               axpy_tile_units<Io, AxpyOne>(), table.entry[nseg].granule_begin);
+  return launch_early(k, l.grid, l.block, true, stream, table, nseg, l.split, a);
+}
+
+cudaError_t launch_axpy_table(const SegTable& table, int nseg, es_dtype_t dtype, uint64_t seed,
+                              float scale, cudaStream_t stream) {
+  AxpyArgs a{};
+  a.seed[0] = philox_sched(seed);
+  a.scale[0] = scale;
+  return dtype == ES_BF16 ? launch_table_io<Bf16Io>(table, nseg, a, stream)
+                          : launch_table_io<F32Io>(table, nseg, a, stream);
 }
 
 cudaError_t launch_axpy_noise2(const PlanView& plan, uint64_t seed, float scale, uint64_t seed2,

@@ -323,7 +323,8 @@ def es_update(plan: Plan, seeds, coeffs, stream=None) -> None:
 def es_perturb_noalloc(segments: Sequence[Segment], dtype: int, seed: int, sigma: float,
                        stream=None) -> None:
     """Perturb (or, with -sigma, restore) without a plan and without any device
-    allocation; the segment table goes to the library's static device array."""
+    allocation; the segment table goes with the launch, or beyond 64 segments to
+    the library's static device array."""
     arr = _seg_array(segments)
     _check(_load().es_perturb_noalloc(arr, len(segments), dtype, seed, sigma, _stream(stream)),
            "es_perturb_noalloc")

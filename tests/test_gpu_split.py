@@ -266,3 +266,23 @@ def test_small_set_update(es, oracle, dtype, numels):
         same((n, "replay"))
     small.close()
     large.close()
+
+
+# es_perturb_noalloc with its table in the launch's parameters (up to 64 segments) and
+# in the static array (65), on a set of one SM's size and on one with long runs.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("nseg,largest", [(1, 9_000_000), (64, 400), (64, 200_000), (65, 400)])
+def test_noalloc_tables(es, dtype, nseg, largest):
+    rng = np.random.default_rng(nseg)
+    tensors = make_params(dtype, [int(n) for n in rng.integers(largest // 2, largest, size=nseg)])
+    twins = [t.clone() for t in tensors]
+    plan, segs = build_plan(es, tensors)
+    segs_b = es.segments_from_tensors(twins, [s.index_base for s in segs])
+    for sigma in (1e-3, -1e-3, 0.05):
+        es.es_perturb(plan, 2**50 + 1, sigma)
+        es.es_perturb_noalloc(segs_b, es.ES_BF16 if dtype == "bf16" else es.ES_FP32, 2**50 + 1,
+                              sigma)
+    torch.cuda.synchronize()
+    for x, y in zip(tensors, twins):
+        assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+    plan.close()
