@@ -1035,8 +1035,8 @@ update_split_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __r
 // group, which may reach beyond [0, n), store element by element.
 // Bound by the generator, and by the stores' bandwidth not far behind (500,000,000
 // aligned floats run at 5.9 TB/s). 50,000,003 floats from an unaligned index 58.8 us
-// (4-byte stores, every block through the general rounds) -> 42.0; 50,000,000
-// aligned 43.8 (256-thread CTAs, one block at a time) -> 36.8, 500,000,000 418 -> 340.
+// (4-byte stores, every block through the general rounds) -> 40.7; 50,000,000
+// aligned 43.8 (256-thread CTAs, one block at a time) -> 36.7, 500,000,000 418 -> 347.
 // 512 to 768 threads and 2 pairs of rows per loop are within 2 %; 1024 threads lose 8 %.
 struct FillArgs {
   PhiloxSched sched;
@@ -1093,7 +1093,6 @@ noise_fill_kernel(const __grid_constant__ FillArgs a, float* __restrict__ out) {
       blockIdx.x * static_cast<uint64_t>(blockDim.x / 32) + threadIdx.x / 32;
   uint64_t m = warp * a.per_warp;
   const uint64_t end = m + a.per_warp < a.groups ? m + a.per_warp : a.groups;
-  wait_for_previous();
   // where the warp's groups that lie inside [0, n) end
   const uint64_t inside = (a.n + a.lead) / 4 < end ? (a.n + a.lead) / 4 : end;
 #pragma unroll 1
@@ -1117,6 +1116,7 @@ noise_fill_kernel(const __grid_constant__ FillArgs a, float* __restrict__ out) {
       const auto gen = sched_gen<true>(a.sched, j_hi);
       Round0 p0 = philox_round0<true>(static_cast<uint32_t>(j) + lane);
       float4* o = reinterpret_cast<float4*>(out + 4 * m - a.lead) + lane;
+      wait_for_previous();
 #pragma unroll 2
       for (uint32_t i = static_cast<uint32_t>(pairs); i > 0; --i) {
         const Round0 rows[2] = {p0, round0_step(p0, 32u)};
@@ -1145,6 +1145,7 @@ noise_fill_kernel(const __grid_constant__ FillArgs a, float* __restrict__ out) {
     }
     const float4 q = fill_group<kShift>(v[0], v[NB - 1], lane);
     const uint64_t k = 4 * (m + lane) - a.lead;  // wraps below zero only in group 0
+    wait_for_previous();
     const float f[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
