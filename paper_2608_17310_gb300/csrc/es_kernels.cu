@@ -60,14 +60,23 @@ struct Bf16Io {
   __device__ static uint4 pack(const float (&f)[8]) {
     return make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
   }
-  // f <- value of round_to_storage(f), element-wise (one rounding to bf16).
-  template <int M>
+  // f <- value of round_to_storage(f), element-wise (one rounding to bf16). kSingly:
+  // with 0 in the low half the converted pair is the rounded value's fp32 bits, one
+  // instruction an element, where packing two and unpacking them takes three for
+  // both: the flip 621 -> 612 us over 792,680,960 parameters. The two-step pass,
+  // which has no register to spare, is faster through the pairs (1093 against 1099).
+  template <bool kSingly, int M>
   __device__ static void round_trip(float (&f)[M]) {
 #pragma unroll
     for (int k = 0; k < M; k += 2) {
-      const uint32_t w = pack2(f[k], f[k + 1]);
-      f[k] = lo(w);
-      f[k + 1] = hi(w);
+      if constexpr (kSingly) {
+        f[k] = __uint_as_float(pack2(0.0f, f[k]));
+        f[k + 1] = __uint_as_float(pack2(0.0f, f[k + 1]));
+      } else {
+        const uint32_t w = pack2(f[k], f[k + 1]);
+        f[k] = lo(w);
+        f[k + 1] = hi(w);
+      }
     }
   }
   // The first `rem` (1 .. 8) elements of the unit at p, the rest zero.
@@ -110,7 +119,7 @@ struct F32Io {
     return make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]),
                       __float_as_uint(f[2]), __float_as_uint(f[3]));
   }
-  template <int M>
+  template <bool, int M>
   __device__ static void round_trip(float (&)[M]) {}
   struct Raw {
     uint4 lo, hi;
@@ -188,7 +197,7 @@ struct Fp8Io {
     return make_uint2(enc2(f[0], f[1]) | (enc2(f[2], f[3]) << 16),
                       enc2(f[4], f[5]) | (enc2(f[6], f[7]) << 16));
   }
-  template <int M>
+  template <bool, int M>
   __device__ static void round_trip(float (&f)[M]) {
 #pragma unroll
     for (int k = 0; k < M; k += 2) {
@@ -440,19 +449,19 @@ __device__ __forceinline__ void axpy_values(const Words& words, const AxpyArgs& 
 #pragma unroll
     for (int k = 0; k < V; ++k) f[k] = add_acc<Io>(f[k], acc[k], inv);
     if constexpr (kPerturb) {
-      Io::round_trip(f);
+      Io::template round_trip<true>(f);
       add_scaled_noise<V>(x, a.scale[kSummed] * inv, f);
     }
   } else if constexpr (Mode::kind == AxpyKind::kFlip) {
     Polar2 pp[V / 4];
     polar_from_words<V / 4>(x, pp);
     apply_noise<V>(pp, a.scale[0] * inv, f);
-    Io::round_trip(f);
+    Io::template round_trip<true>(f);
     apply_noise<V>(pp, a.scale[1] * inv, f);
   } else {
     add_scaled_noise<V>(x, a.scale[0] * inv, f);
     if constexpr (kSeeds == 2) {
-      Io::round_trip(f);
+      Io::template round_trip<false>(f);
       words(1, x);
       add_scaled_noise<V>(x, a.scale[1] * inv, f);
     }
@@ -481,7 +490,7 @@ struct AxpyGens {
 // loop body run 6-15 % faster than 2 or 3 CTAs of 256 threads on a body of four
 // vectors. Measured on sm_103a over 792,680,960 parameters (us; 256 threads, 4
 // vectors, 1 ahead, grid-stride tiles -> this): bf16 one step 678 -> 569 (5.58 TB/s),
-// two steps 1217 -> 1094 (1.449e12 Gaussians/s), flip 729 -> 621; fp32 971 -> 960 (6.6
+// two steps 1217 -> 1093 (1.450e12 Gaussians/s), flip 729 -> 612; fp32 971 -> 960 (6.6
 // TB/s: HBM), 1366 -> 1077, 976 -> 961; FP8 636 -> 570, 1301 -> 1118, 718 -> 635 (8
 // elements at a time: 16 hold twice the registers and body, and cost the sums of 4 and
 // more seeds 1-10 %).
@@ -1206,7 +1215,7 @@ struct GridEntry {
   int device;
   int ctas;
 };
-constexpr int kGridCacheSize = 128;
+constexpr int kGridCacheSize = 512;
 std::mutex g_grid_mutex;
 GridEntry g_grid_cache[kGridCacheSize];
 int g_grid_used = 0;
