@@ -1,4 +1,4 @@
-// Internal interface between the C-ABI host layer (es_host.cpp) and the CUDA
+// Internal interface between the C-ABI host layer (es_host.cu) and the CUDA
 // kernels (es_kernels.cu). Not part of the public ABI.
 #pragma once
 
@@ -24,6 +24,7 @@ constexpr int kBlockThreads = 256;
 
 // Bytes per element, per dtype.
 constexpr size_t dtype_bytes(es_dtype_t dt) { return dt == ES_FP8_E4M3 ? 1u : dt == ES_BF16 ? 2u : 4u; }
+
 // Device-side segment descriptor. A plan's table has nseg + 1 entries; the
 // last is a sentinel whose granule_begin is the total number of granules.
 struct SegDesc {

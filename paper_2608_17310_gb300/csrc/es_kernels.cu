@@ -269,7 +269,7 @@ __device__ __forceinline__ void polar_from_words(const uint4 (&x)[NB], Polar2 (&
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     xa[b] = make_uint2(x[b].x, x[b].z);
-    p[b] = polar2_sq<true>(x[b]);
+    p[b] = polar2_sq(x[b]);
   }
   fix_near_one<NB>(xa, p);
 #pragma unroll

@@ -34,11 +34,10 @@ __host__ __device__ inline PhiloxKey philox_key(uint64_t seed) {
 // High and low words of the 32x32->64-bit product m * x. Two forms, with the
 // same words: two 32-bit multiplies (mul.hi.u32, mul.lo.u32), or one multiply
 // with a 64-bit result (mul.wide.u32). Measured on sm_103a in the library's
-// kernels, the fastest mix is the 64-bit form in the eight full rounds of the
-// per-tile path (philox_block_tile) and the 32-bit pair everywhere else (the
-// first two rounds, the per-tile constants and the general path): 5-8 %
-// faster than either form throughout, which cost registers and occupancy in
-// the fused update.
+// kernels, the fastest mix is the 64-bit form in the eight full rounds and the
+// 32-bit pair everywhere else (the first two rounds, the constants of a high
+// counter word and the general path): 5-8 % faster than either form throughout;
+// the one-step pass takes the 64-bit form in every round.
 __device__ __forceinline__ uint32_t mul_hi(uint32_t m, uint32_t x) { return __umulhi(m, x); }
 __device__ __forceinline__ uint32_t mul_lo(uint32_t m, uint32_t x) { return m * x; }
 __device__ __forceinline__ void mul_wide(uint32_t m, uint32_t x, uint32_t& hi, uint32_t& lo) {
@@ -308,22 +307,11 @@ struct Polar {
   float r, c, s;
 };
 
-// The pair before the square root: .r holds radius^2, from radius_sq (kLogOnly
-// false) or from the hardware log2 alone (kLogOnly true; the caller then
-// replaces the near-one inputs' radius^2 by radius_sq_series).
-template <bool kLogOnly>
-__device__ __forceinline__ Polar polar_sq(uint32_t xa, uint32_t xb) {
+__device__ __forceinline__ Polar polar(uint32_t xa, uint32_t xb) {
   Polar p;
-  const float u = uniform_open(xa);
-  p.r = kLogOnly ? radius_sq_log(u) : radius_sq(u);
+  p.r = sqrt_approx(radius_sq(uniform_open(xa)));
   const float f = one_plus_top23(xb);
   sincos_approx(fmaf(f, kTwoPi, kAngleOffset), &p.s, &p.c);
-  return p;
-}
-
-__device__ __forceinline__ Polar polar(uint32_t xa, uint32_t xb) {
-  Polar p = polar_sq<false>(xa, xb);
-  p.r = sqrt_approx(p.r);
   return p;
 }
 
@@ -337,35 +325,20 @@ struct Polar2 {
   float2 r, c, s;
 };
 
-// Both pairs before their square roots (.r holds radius^2), as polar_sq.
-template <bool kLogOnly>
+// Both pairs before their square roots: .r holds radius^2 from the hardware log2
+// alone; the caller then replaces the near-one inputs' (fix_near_one).
 __device__ __forceinline__ Polar2 polar2_sq(const uint4& x) {
   Polar2 p;
   const float2 fa = make_float2(one_plus_top23(x.x), one_plus_top23(x.z));
   const float kHalfUlpBelowOne = __uint_as_float(0x3F7FFFFFu);
   const float2 u = __fadd2_rn(fa, make_float2(-kHalfUlpBelowOne, -kHalfUlpBelowOne));
-  const float2 logged =
-      __fmul2_rn(make_float2(log2_approx(u.x), log2_approx(u.y)),
-                 make_float2(kMinusTwoLn2, kMinusTwoLn2));
-  if constexpr (kLogOnly) {
-    p.r = logged;
-  } else {
-    const float2 t = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(-u.x, -u.y));
-    const float2 series = __ffma2_rn(t, t, __fadd2_rn(t, t));
-    p.r.x = u.x > kNearOne ? series.x : logged.x;
-    p.r.y = u.y > kNearOne ? series.y : logged.y;
-  }
+  p.r = __fmul2_rn(make_float2(log2_approx(u.x), log2_approx(u.y)),
+                   make_float2(kMinusTwoLn2, kMinusTwoLn2));
   const float2 fb = make_float2(one_plus_top23(x.y), one_plus_top23(x.w));
   const float2 ang = __ffma2_rn(fb, make_float2(kTwoPi, kTwoPi),
                                 make_float2(kAngleOffset, kAngleOffset));
   sincos_approx(ang.x, &p.s.x, &p.c.x);
   sincos_approx(ang.y, &p.s.y, &p.c.y);
-  return p;
-}
-
-__device__ __forceinline__ Polar2 polar2(const uint4& x) {
-  Polar2 p = polar2_sq<false>(x);
-  p.r = make_float2(sqrt_approx(p.r.x), sqrt_approx(p.r.y));
   return p;
 }
 

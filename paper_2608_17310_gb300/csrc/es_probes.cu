@@ -361,7 +361,7 @@ probe_kernel(int iters, uint32_t seed, unsigned long long* __restrict__ rec,
       for (int b = 0; b < 2; ++b) {
         const uint4 x = esopt::philox_block_rk<false>(j + b, tc, ps.rk[1], ps.rk[2], ps.rk + 4);
         xa[b] = make_uint2(x.x, x.z);
-        p[b] = esopt::polar2_sq<true>(x);
+        p[b] = esopt::polar2_sq(x);
       }
       esopt::fix_near_one<2>(xa, p);
 #pragma unroll
@@ -395,7 +395,7 @@ probe_kernel(int iters, uint32_t seed, unsigned long long* __restrict__ rec,
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         xa[b] = make_uint2(x[b].x, x[b].z);
-        p[b] = esopt::polar2_sq<true>(x[b]);
+        p[b] = esopt::polar2_sq(x[b]);
       }
       esopt::fix_near_one<2>(xa, p);
 #pragma unroll
@@ -467,7 +467,7 @@ probe_kernel(int iters, uint32_t seed, unsigned long long* __restrict__ rec,
         // the slot is free again; its last use needs no release
         if (i + kSplitStages < iters) mbar_arrive(&empty_bar[st][pair]);
         uint2 xa[2] = {make_uint2(x0.x, x0.z), make_uint2(x1.x, x1.z)};
-        esopt::Polar2 p[2] = {esopt::polar2_sq<true>(x0), esopt::polar2_sq<true>(x1)};
+        esopt::Polar2 p[2] = {esopt::polar2_sq(x0), esopt::polar2_sq(x1)};
         esopt::fix_near_one<2>(xa, p);
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
