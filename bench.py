@@ -812,8 +812,8 @@ def _rates(P, gaussians_per_param, bytes_total, ms, peaks_):
 
 
 def run_replay(args, rank, world, dist):
-    """es_replay of K logged generations (N seeds each) in one pass over the
-    parameters, against the same K generations as K es_update calls."""
+    """es_replay of K logged generations (N seeds each) against the same K
+    generations as K es_update calls."""
     import torch
     from paper_2608_17310_gb300 import build, esopt as es
 
@@ -837,13 +837,15 @@ def run_replay(args, rank, world, dist):
                                           es.ES_SCALE_PAPER))
     all_seeds, all_coeffs = np.concatenate(seeds), np.concatenate(coeffs)
     counts = np.full(K, n, dtype=np.int32)
-    # launches es_replay makes: generations of fewer than 4 non-zero seeds
-    # share a pass (<= ES_MAX_SEEDS seeds, <= 256 generations); a larger one
-    # has a pass of its own; passes break only between generations
+    # launches es_replay makes: on plans of 2^25 parameters and more a generation
+    # has a pass of its own (in fp32 from 2 non-zero seeds on); the others share
+    # passes (<= ES_MAX_SEEDS seeds, <= 256 generations), which break only between
+    # generations
+    own_from = 2 if esize == 4 else 1
     passes, in_pass, gens = 0, 0, 0
     for g in range(K):
         nz = int(np.count_nonzero(coeffs[g]))
-        own = nz >= 4
+        own = P >= 1 << 25 and nz >= own_from
         if nz and gens and (own or in_pass + nz > es.ES_MAX_SEEDS or gens == 256):
             passes, in_pass, gens = passes + 1, 0, 0
         if nz:

@@ -49,6 +49,9 @@
  *     repeated calls give bit-identical parameters on every run.
  *   - Thread safety: distinct plans may be used from different threads; one plan
  *     must not be used on two streams at once.
+ *   - Stream order holds as usual. Kernels are launched so that one may begin
+ *     while the kernel before it in its stream is still ending; it reads its own
+ *     tables and touches no caller memory until that one has completed.
  *   - Plan-based device entry points neither synchronise the host nor allocate
  *     per call, so they can be recorded in a CUDA graph (stream capture); the
  *     host arguments of a captured call (seeds, coefficients, sigma) are fixed

@@ -357,10 +357,9 @@ def _sample(segs, rng, per_seg=2048, edge=64):
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_replay_matches_oracle_generation_by_generation(es, oracle, dtype):
     # The seed log of a run is replayed from the base parameters (App. D.2-D.4):
-    # 400 logged generations. The first 300 have 1..3 seeds, so they share
-    # passes over theta and pass the 256-generation limit of one pass; the
-    # last 100 have 1..8 seeds, so generations of 4 or more get passes of their
-    # own through the single-generation kernel. Some generations and some
+    # 400 logged generations of 1..3 and then 1..8 seeds: on a set of this size
+    # they share passes over theta and pass the 256-generation limit of one pass.
+    # Some generations and some
     # coefficients are zero. The oracle applies the same generations one by one
     # in double precision, rounding to storage after each, from the same start.
     numels = [9, 8193, 20000, 4096 * 3 + 5]
