@@ -8,7 +8,8 @@
 // SM gets the same work whatever the set's size and however it is divided into
 // tensors.
 // Every element is owned by exactly one thread: no atomics, no shared state
-// between threads except the staged seeds of the update.
+// between threads except the staged seeds of the update and, on small sets, the
+// polar forms that its warps hand over.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -528,8 +529,8 @@ __host__ __device__ constexpr uint64_t axpy_tile_units() {
 
 // `tiles` whole tiles of one segment, all with the same high counter word,
 // from the calling thread's first vector at p, whose first Philox block is
-// j_thread. Vector u of a tile is one 16-byte vector per thread, so each load
-// and store instruction of a warp covers 512 contiguous bytes; the load of the
+// j_thread. Vector u of a tile is one 16-byte vector per thread (FP8: 8 bytes), so
+// each load and store instruction of a warp covers 512 (256) contiguous bytes; the load of the
 // vector `ahead` of the current one is issued before that is computed. Round 0's Philox
 // product (of the counter alone) is stepped by 64-bit additions from the
 // thread's first block instead of multiplied.
@@ -598,9 +599,9 @@ __device__ __forceinline__ void axpy_unit(const UnitRef<Io>& r, const AxpyArgs& 
   Io::store_unit(r.p, r.rem, Io::pack_unit(f));
 }
 
-// theta[g] <- round(theta[g] + scale * eps_seed[g]) over every segment, or the
-// two steps of kTwo and kFlip. For a scaled storage type (FP8) the noise is
-// added in units of the segment's scale: scale * inv_scale[segment].
+// theta[g] <- round(theta[g] + scale * eps_seed[g]) over every segment, or what
+// else Mode says. For a scaled storage type (FP8) the noise is added in units of
+// the segment's scale: scale * inv_scale[segment].
 // A CTA alternates between runs of whole tiles inside one segment (axpy_run)
 // and up to a tile's worth of units wherever a segment, the range or a high
 // counter word ends (axpy_unit; each thread finds its unit's segment). It waits for
@@ -855,7 +856,7 @@ __device__ __forceinline__ void update_unit(typename Io::Scalar* p, int rem, flo
 // parameters (ms; 3 CTAs of 256 threads on grid-stride tiles -> one CTA of 640):
 // 8 seeds bf16 4.70 -> 4.43 (1.43e12 Gaussians/s), fp32 5.32 -> 4.42 and FP8
 // 4.90 -> 4.41 (their seed loops were not pipelined: they took 8 elements in another form), 16 seeds +
-// perturb bf16 9.77 -> 9.20, 2 seeds bf16 1.48 -> 1.30. Several generations run fastest
+// perturb bf16 9.77 -> 9.15. Several generations run fastest
 // with 768: 8 generations of 2 seeds 10.59 -> 9.41.
 template <bool kSingle>
 __host__ __device__ constexpr int update_threads() {
@@ -939,7 +940,7 @@ update_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restric
 // element of a block, which add them up in ascending seed order with the same
 // operations as update_unit, so the values are the same bits. What bounds it is
 // latency: n / kWarps rounds of one block's generation instead of n of two blocks'.
-// 65,536 fp32 parameters, us in a graph (update_unit's or the sums' pass -> this):
+// 65,536 fp32 parameters, us in a graph (the seed loop's or the sums' pass -> this):
 // 1 seed 1.7 -> 1.6, 8 seeds 3.0 -> 2.1, 32 seeds 6.9 -> 5.8, 128 seeds 21.9 -> 20.0;
 // 1024 parameters 32 seeds 6.8 -> 2.5. It generates one block per thread where
 // update_unit overlaps two, so it loses once the GPU is full: 98,304 parameters, 8
