@@ -17,6 +17,7 @@ import ctypes
 import os
 import sys
 from dataclasses import dataclass
+from types import SimpleNamespace
 from typing import Iterable, Sequence
 
 import numpy as np
@@ -71,10 +72,6 @@ def _load() -> ctypes.CDLL:
     vp, u64, f32, f64, i32 = (ctypes.c_void_p, ctypes.c_uint64, ctypes.c_float,
                               ctypes.c_double, ctypes.c_int)
     P = ctypes.POINTER
-    # numeric arrays go by address (_addr): a typed ctypes pointer takes 2-3 us to
-    # build, and small calls are bound by their host time (es_update of a set that
-    # one SM holds: 14.5 us a call with typed pointers and a Stream object, 6.2 us so)
-    arr = vp
     sigs = {
         "es_plan_create": (i32, [P(es_segment_t), i32, i32, P(vp)]),
         "es_plan_create_scaled": (i32, [P(es_segment_t), P(f32), i32, i32, P(vp)]),
@@ -87,13 +84,13 @@ def _load() -> ctypes.CDLL:
         "es_perturb": (i32, [vp, u64, f32, vp]),
         "es_restore": (i32, [vp, u64, f32, vp]),
         "es_restore_perturb": (i32, [vp, u64, f32, u64, f32, vp]),
-        "es_update": (i32, [vp, arr, arr, i32, vp]),
-        "es_update_perturb": (i32, [vp, arr, arr, i32, u64, f32, vp]),
-        "es_replay": (i32, [vp, arr, arr, arr, i32, vp]),
-        "es_normalize_rewards": (i32, [arr, i32, f64, arr]),
+        "es_update": (i32, [vp, P(u64), P(f32), i32, vp]),
+        "es_update_perturb": (i32, [vp, P(u64), P(f32), i32, u64, f32, vp]),
+        "es_replay": (i32, [vp, P(u64), P(f32), P(i32), i32, vp]),
+        "es_normalize_rewards": (i32, [P(f64), i32, f64, P(f64)]),
         "es_sigma_cosine": (f64, [f64, f64, i32, i32]),
-        "es_update_coeffs": (i32, [arr, i32, f64, f64, i32, arr]),
-        "es_fold_antithetic": (i32, [arr, arr, i32, f64, f64, i32, arr]),
+        "es_update_coeffs": (i32, [P(f64), i32, f64, f64, i32, P(f32)]),
+        "es_fold_antithetic": (i32, [P(f64), P(f64), i32, f64, f64, i32, P(f32)]),
         "es_perturb_noalloc": (i32, [P(es_segment_t), i32, i32, u64, f32, vp]),
         "es_status_string": (ctypes.c_char_p, [i32]),
         "es_last_error": (ctypes.c_char_p, []),
@@ -102,6 +99,19 @@ def _load() -> ctypes.CDLL:
         fn = getattr(L, name)
         fn.restype = res
         fn.argtypes = args
+    # The functions of this module pass numeric arrays, whose type they have made
+    # sure of, by address (_addr): a typed ctypes pointer takes 2-3 us to build, and
+    # small calls are bound by their host time (es_update of a set that one SM holds:
+    # 14.5 us a call with typed pointers and a Stream object, 6.2 us so). L[name] is a
+    # function object of its own, so a caller of lib() keeps the typed ones.
+    L.by_address = SimpleNamespace()
+    for name in ("es_update", "es_update_perturb", "es_replay", "es_normalize_rewards",
+                 "es_update_coeffs", "es_fold_antithetic"):
+        res, args = sigs[name]
+        fn = L[name]
+        fn.restype = res
+        fn.argtypes = [vp if a in (P(u64), P(f32), P(f64), P(i32)) else a for a in args]
+        setattr(L.by_address, name, fn)
     _lib = L
     return L
 
@@ -316,8 +326,8 @@ def es_update(plan: Plan, seeds, coeffs, stream=None) -> None:
     c = np.ascontiguousarray(coeffs, dtype=np.float32)
     if s.size != c.size:
         raise ValueError("seeds and coeffs differ in length")
-    _check(_load().es_update(plan.handle, _addr(s), _addr(c), s.size, _stream(stream)),
-           "es_update")
+    _check(_load().by_address.es_update(plan.handle, _addr(s), _addr(c), s.size,
+                                        _stream(stream)), "es_update")
 
 
 def es_perturb_noalloc(segments: Sequence[Segment], dtype: int, seed: int, sigma: float,
@@ -336,8 +346,9 @@ def es_update_perturb(plan: Plan, seeds, coeffs, next_seed: int, sigma_next: flo
     c = np.ascontiguousarray(coeffs, dtype=np.float32)
     if s.size != c.size:
         raise ValueError("seeds and coeffs differ in length")
-    _check(_load().es_update_perturb(plan.handle, _addr(s), _addr(c), s.size, next_seed,
-                                     sigma_next, _stream(stream)), "es_update_perturb")
+    _check(_load().by_address.es_update_perturb(plan.handle, _addr(s), _addr(c), s.size, next_seed,
+                                                sigma_next, _stream(stream)),
+           "es_update_perturb")
 
 
 def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
@@ -347,8 +358,8 @@ def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
     n = np.ascontiguousarray(counts, dtype=np.int32)
     if s.size != c.size or int(n.sum()) != s.size:
         raise ValueError("seeds, coeffs and counts do not agree")
-    _check(_load().es_replay(plan.handle, _addr(s), _addr(c), _addr(n), n.size, _stream(stream)),
-           "es_replay")
+    _check(_load().by_address.es_replay(plan.handle, _addr(s), _addr(c), _addr(n), n.size,
+                                        _stream(stream)), "es_replay")
 
 
 # --- host-side generation control ---------------------------------------------------
@@ -356,7 +367,7 @@ def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
 def es_normalize_rewards(rewards, eps_z: float = 1e-8) -> np.ndarray:
     r = _f64(rewards)
     out = np.empty_like(r)
-    _check(_load().es_normalize_rewards(_addr(r), r.size, eps_z, _addr(out)),
+    _check(_load().by_address.es_normalize_rewards(_addr(r), r.size, eps_z, _addr(out)),
            "es_normalize_rewards")
     return out
 
@@ -368,7 +379,7 @@ def es_sigma_cosine(sigma0: float, sigmaT: float, t: int, T: int) -> float:
 def es_update_coeffs(rhat, alpha: float, sigma: float, mode: int = ES_SCALE_PAPER) -> np.ndarray:
     r = _f64(rhat)
     out = np.empty(r.size, dtype=np.float32)
-    _check(_load().es_update_coeffs(_addr(r), r.size, alpha, sigma, mode, _addr(out)),
+    _check(_load().by_address.es_update_coeffs(_addr(r), r.size, alpha, sigma, mode, _addr(out)),
            "es_update_coeffs")
     return out
 
@@ -379,6 +390,6 @@ def es_fold_antithetic(rhat_pos, rhat_neg, alpha: float, sigma: float,
     if p.size != m.size:
         raise ValueError("rhat_pos and rhat_neg differ in length")
     out = np.empty(p.size, dtype=np.float32)
-    _check(_load().es_fold_antithetic(_addr(p), _addr(m), p.size, alpha, sigma, mode, _addr(out)),
-           "es_fold_antithetic")
+    _check(_load().by_address.es_fold_antithetic(_addr(p), _addr(m), p.size, alpha, sigma, mode,
+                                                 _addr(out)), "es_fold_antithetic")
     return out

@@ -186,6 +186,34 @@ def test_normalize_rewards_in_place(E, oracle):
     assert np.allclose(buf, want, rtol=1e-14, atol=1e-14)
 
 
+def test_raw_functions_refuse_arrays_of_another_type(E):
+    # A caller of lib() that passes an array of another element type is refused
+    # before the call: the library would read or write it out of range.
+    import ctypes
+    f32 = (ctypes.c_float * 4)()
+    f64 = (ctypes.c_double * 4)()
+    u64 = (ctypes.c_uint64 * 4)()
+    i32 = (ctypes.c_int * 4)()
+    i16 = (ctypes.c_int16 * 4)()
+    L = E.lib()
+    bad = [
+        lambda: L.es_update(None, i32, f32, 4, None),
+        lambda: L.es_update(None, u64, f64, 4, None),
+        lambda: L.es_update_perturb(None, u64, f64, 4, 1, 1e-3, None),
+        lambda: L.es_replay(None, u64, f32, i16, 4, None),
+        lambda: L.es_normalize_rewards(f32, 4, 1e-8, f64),
+        lambda: L.es_normalize_rewards(f64, 4, 1e-8, f32),
+        lambda: L.es_update_coeffs(f64, 4, 1e-3, 1e-3, 0, f64),
+        lambda: L.es_fold_antithetic(f64, f32, 4, 1e-3, 1e-3, 0, f32),
+        lambda: L.es_update(None, u64, 4096, 4, None),
+    ]
+    for call in bad:
+        with pytest.raises(ctypes.ArgumentError):
+            call()
+    assert L.es_normalize_rewards(f64, 4, 1e-8, f64) == E.ES_OK
+    assert L.es_update_coeffs(f64, 4, 1e-3, 1e-3, 0, f32) == E.ES_OK
+
+
 def test_assign_index_bases_overflow_returns_zero(E):
     segs = [E.Segment(0, 2**63), E.Segment(0, 2**63 + 16)]
     assert E.es_assign_index_bases(segs) == 0
