@@ -231,8 +231,7 @@ def es_assign_index_bases(segments: Sequence[Segment]) -> int:
 def es_plan_create(segments: Sequence[Segment], dtype: int, keepalive: Iterable = ()) -> Plan:
     arr = _seg_array(segments)
     handle = ctypes.c_void_p()
-    _check(_load().es_plan_create(arr, len(segments), dtype,
-        ctypes.byref(handle)),
+    _check(_load().es_plan_create(arr, len(segments), dtype, ctypes.byref(handle)),
            "es_plan_create")
     return Plan(handle.value, int(_load().es_plan_numel(handle)), dtype, keepalive)
 
@@ -245,9 +244,8 @@ def es_plan_create_scaled(segments: Sequence[Segment], scales, dtype: int,
     if sc.size != len(segments):
         raise ValueError("one scale per segment")
     handle = ctypes.c_void_p()
-    _check(_load().es_plan_create_scaled(
-        arr, sc.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), len(segments), dtype,
-        ctypes.byref(handle)),
+    _check(_load().es_plan_create_scaled(arr, sc.ctypes.data_as(ctypes.POINTER(ctypes.c_float)),
+                                         len(segments), dtype, ctypes.byref(handle)),
            "es_plan_create_scaled")
     return Plan(handle.value, int(_load().es_plan_numel(handle)), dtype, keepalive, sc)
 
