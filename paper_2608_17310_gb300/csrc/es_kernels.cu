@@ -20,21 +20,6 @@
 
 #include "es_internal.h"
 #include "es_noise.cuh"
-#if FX==0
-#define FSH 1024,2,2
-#elif FX==1
-#define FSH 768,2,2
-#elif FX==2
-#define FSH 896,2,2
-#elif FX==3
-#define FSH 768,1,1
-#elif FX==4
-#define FSH 768,3,3
-#elif FX==5
-#define FSH 640,2,2
-#elif FX==6
-#define FSH 640,1,1
-#endif
 
 namespace esopt {
 namespace {
