@@ -244,6 +244,10 @@ es_status_t create_plan(const es_segment_t* segs, const float* scales, int nseg,
     err = cudaMemcpy(plan->d_inv_scale, inv.data(), inv.size() * sizeof(float),
                      cudaMemcpyHostToDevice);
   }
+  // From pageable memory cudaMemcpy may return once the source has been staged, and
+  // a stream that does not synchronise with the legacy one would not wait for the
+  // rest: the plan is handed out when its table is on the device.
+  if (err == cudaSuccess) err = cudaStreamSynchronize(cudaStreamLegacy);
   if (err != cudaSuccess) {
     cudaFree(plan->d_segs);
     delete plan;

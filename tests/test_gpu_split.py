@@ -210,6 +210,36 @@ def test_launches_behind_other_work(es, numel):
     plan.close()
 
 
+# A plan is ready on every stream when it is handed out: used at once on a stream
+# that does not synchronise with the default one and is still busy, its table (and
+# FP8's scales) are those of the same call on a plan made long before.
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+def test_new_plan_on_a_busy_stream(es, dtype):
+    n, pieces = 1 << 20, 900
+    if dtype == "fp8":
+        codes = np.random.default_rng(8).integers(0, 120, size=n).astype(np.uint8)
+        a = torch.from_numpy(codes).cuda()
+    else:
+        (a,) = make_params("bf16", [n], seed=8)
+    b, busy = a.clone(), torch.randn(1 << 24, device="cuda")
+    step = n // pieces // 16 * 16
+    bases = list(range(0, step * pieces, step))
+    scales = [2.0**-9 * (1 + k % 7) for k in range(pieces)] if dtype == "fp8" else None
+    old = es.plan_from_tensors([b[o:o + step] for o in bases], bases, scales)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    for k in range(8):
+        with torch.cuda.stream(side):
+            busy.mul_(1.0)
+            new = es.plan_from_tensors([a[o:o + step] for o in bases], bases, scales)
+            es.es_perturb(new, k, 1e-3)
+            es.es_perturb(old, k, 1e-3)
+        torch.cuda.synchronize()
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), k
+        new.close()
+    old.close()
+
+
 # The update of a small set, whose seeds are spread over warps: the same bits as
 # in a plan that a further, larger tensor takes out of that range, and equal to the
 # oracle; counts at the edges of a round of 8 and of 32 seeds, sets on both sides of
