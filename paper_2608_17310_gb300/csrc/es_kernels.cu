@@ -1037,11 +1037,13 @@ struct FillArgs {
   PhiloxSched sched;
   uint64_t j_first;   // block of group 0 (kShift > 0: the block it ends in)
   uint64_t groups;
-  uint64_t per_warp;  // groups of one warp: 32, or a multiple of 64
+  uint64_t per_warp;  // groups of one warp: a row, or a multiple of 64
   uint64_t n;
   int lead;
 };
 constexpr int kFillThreads = 768;
+// Groups of a row on its own (noise_row_kernel).
+__host__ __device__ constexpr uint64_t fill_row_groups(int shift) { return shift != 0 ? 31 : 32; }
 
 __device__ __forceinline__ float4 polar_values(const Polar2& p) {
   const float2 lo = __fmul2_rn(make_float2(-p.r.x, -p.r.x), make_float2(p.c.x, p.s.x));
@@ -1146,6 +1148,39 @@ noise_fill_kernel(const __grid_constant__ FillArgs a, float* __restrict__ out) {
     for (int i = 0; i < 4; ++i)
       if (m + lane < end && k + i < a.n) out[k + i] = f[i];
     m += 32;
+  }
+  let_next_start();
+}
+
+// The same where one row per warp is enough for `out` (2 CTAs per SM: 933,888 aligned
+// floats), each lane with its own high word and bounds. With a shift lane 0 generates
+// the block before the row's first, for lane 1, and has no group of its own;
+// noise_fill_kernel has every lane generate that block, which cost unaligned fills of
+// this size more than one thread per block had. Bound by one block's latency and the
+// launch. In a graph, us (one thread per block; noise_fill_kernel -> this): unaligned
+// 1 float 0.87; 1.24 -> 0.83, 450,000 1.65; 2.10 -> 1.36, 800,000 2.22; 2.38 -> 1.85;
+// aligned 450,000 1.90; 1.61 -> 1.24.
+template <int kShift>
+__global__ void __launch_bounds__(kFillThreads)
+noise_row_kernel(const __grid_constant__ FillArgs a, float* __restrict__ out) {
+  constexpr uint32_t kBefore = kShift != 0 ? 1 : 0;
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t warp =
+      blockIdx.x * static_cast<uint64_t>(blockDim.x / 32) + threadIdx.x / 32;
+  const uint64_t m = warp * fill_row_groups(kShift);
+  if (m < a.groups) {
+    const uint64_t group = m + lane - kBefore, j = a.j_first + group;
+    const auto gen = sched_gen<false>(a.sched, static_cast<uint32_t>(j >> 32));
+    const Round0 p0[1] = {philox_round0<false>(static_cast<uint32_t>(j))};
+    float4 v[1];
+    fill_values<1>(gen, p0, v);
+    const float4 q = fill_group<kShift>(v[0], v[0], lane);
+    const uint64_t k = 4 * group - a.lead;  // wraps below zero only in group 0
+    wait_for_previous();
+    const float f[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if ((kShift == 0 || lane > 0) && group < a.groups && k + i < a.n) out[k + i] = f[i];
   }
   let_next_start();
 }
@@ -1464,16 +1499,26 @@ cudaError_t launch_noise_fill(uint64_t seed, uint64_t index_base, uint64_t n, fl
               (shift != 0 ? 1u : 0u);
   a.groups = n / 4 + (n % 4 + a.lead + 3) / 4;
   using Kernel = void (*)(FillArgs, float*);
-  static constexpr Kernel kKernels[4] = {noise_fill_kernel<0>, noise_fill_kernel<1>,
-                                         noise_fill_kernel<2>, noise_fill_kernel<3>};
-  const Kernel k = kKernels[shift];
+  static constexpr Kernel kRow[4] = {noise_row_kernel<0>, noise_row_kernel<1>, noise_row_kernel<2>,
+                                     noise_row_kernel<3>};
+  static constexpr Kernel kFill[4] = {noise_fill_kernel<0>, noise_fill_kernel<1>,
+                                      noise_fill_kernel<2>, noise_fill_kernel<3>};
   int dev = 0;
   cudaGetDevice(&dev);
-  const uint64_t ctas =
-      static_cast<uint64_t>(resident_ctas(reinterpret_cast<const void*>(k), kFillThreads, dev));
-  const uint64_t most = ctas * (kFillThreads / 32);  // warps
-  const uint64_t rows = ((a.groups + 31) / 32 + most - 1) / most;
-  a.per_warp = rows == 1 ? 32 : (rows + 1) / 2 * 64;
+  auto resident = [&](Kernel k) {
+    return static_cast<uint64_t>(
+        resident_ctas(reinterpret_cast<const void*>(k), kFillThreads, dev));
+  };
+  constexpr uint64_t kWarps = kFillThreads / 32;
+  Kernel k = kRow[shift];
+  uint64_t ctas = resident(k);
+  a.per_warp = fill_row_groups(shift);
+  if ((a.groups + a.per_warp - 1) / a.per_warp > ctas * kWarps) {
+    k = kFill[shift];
+    ctas = resident(k);
+    const uint64_t rows = ((a.groups + 31) / 32 + ctas * kWarps - 1) / (ctas * kWarps);
+    a.per_warp = (rows + 1) / 2 * 64;
+  }
   const uint64_t warps = (a.groups + a.per_warp - 1) / a.per_warp;
   // spread over the SMs, whole sets of 4 warps (one per SM sub-partition) above 4
   uint64_t per_cta = (warps + ctas - 1) / ctas;

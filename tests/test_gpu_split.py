@@ -107,8 +107,8 @@ def test_long_runs_equal_short_segments(es, oracle, dtype, numel):
 
 
 # es_noise_fill for every way that index_base and out's 16-byte alignment can
-# meet: the smallest counts, the edges of a row of 32 groups and of a pair of
-# rows, and counts that fill every warp, across the change of the high counter
+# meet: the smallest counts, the edges of a row of 31 or 32 groups and of a pair of
+# rows, and counts that fill every warp once and more often, across the change of the high counter
 # word; bit-identical to one aligned fill, which the oracle checks.
 @pytest.mark.parametrize("lead", [0, 1, 2, 3])
 def test_noise_fill_alignments(es, oracle, lead):
@@ -121,7 +121,8 @@ def test_noise_fill_alignments(es, oracle, lead):
     assert np.all(np.abs(got - want) <= 1e-5 * np.maximum(1.0, np.abs(want)))
     out = torch.empty(3_000_032, device="cuda")
     for skip in (0, 1, 2, 3, 3_998):
-        for n in (1, 2, 3, 4, 5, 127, 128, 129, 255, 256, 257, 4_001, 622_593, 3_000_001):
+        for n in (1, 2, 3, 4, 5, 123, 124, 125, 127, 128, 129, 255, 256, 257, 4_001, 300_001,
+                  452_353, 622_593, 904_703, 904_704, 904_705, 933_889, 3_000_001):
             if skip + n > whole.numel():
                 continue
             out.fill_(7.0)
