@@ -661,6 +661,49 @@ axpy_noise_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __res
   axpy_pass<Io, Mode>(segs, nseg, inv_scale, split, a);
 }
 
+// The same where every CTA's range is one row at most, one unit per thread: a thread
+// has its unit's place before it waits, so that theta's load is all that follows the
+// wait. Lane l of a warp loads where segment lo + l begins (a row's 32 units touch at
+// most 17 segments) and the threads bisect that by shuffles, which leaves two or three
+// dependent loads of the table. axpy_pass looks a row of several segments up behind the
+// wait, so a graph of passes over 2 to 4 small tensors ran slower there than through a
+// walk along the table, though passes in a stream did not.
+// Bound by the latency of one pass. In a graph, us (a walk along the table; axpy_pass ->
+// this): 2 fp32 tensors of 300,000 at most, two steps 1.98; 2.39 -> 1.49, perturb 2.06;
+// 2.06 -> 1.36; 2 bf16 ones 2.14; 2.43 -> 1.69 and 2.02; 2.14 -> 1.45; 900 bf16 ones of
+// 6,000 at most, two steps 3.25 -> 2.27.
+// One segment has no lookup to move: up to kRowGranules, where a CTA has 4 warps at
+// most, this is the faster one (65,536 fp32 parameters, two steps 2.02 -> 1.36, perturb
+// 1.73 -> 1.16); above, a CTA of the next pass that starts early beside one of this pass
+// loads some SMs twice, and it is between 20 % faster and 16 % slower (200,000 fp32
+// parameters, perturb 1.49 -> 1.73), so one larger segment stays with axpy_pass.
+constexpr uint64_t kRowGranules = 8192;
+template <class Io, class Mode>
+__global__ void __launch_bounds__(axpy_shape<Io, Mode>().threads)
+axpy_row_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restrict__ inv_scale,
+                const Split split, const __grid_constant__ AxpyArgs a) {
+  const int lane = static_cast<int>(threadIdx.x & 31u);
+  const uint64_t last = range_end(split) - 1;
+  const uint64_t unit = range_begin(split) * kUnitsPerGranule + threadIdx.x;
+  const uint64_t granule = unit / kUnitsPerGranule;
+  const uint64_t mine = granule < last ? granule : last;
+  int s = 0;
+  if (nseg > 1) {
+    const uint64_t warp_first = __shfl_sync(0xFFFFFFFFu, mine, 0);
+    const int lo = nseg > 32 ? search_segment(segs, 0, nseg, warp_first) : 0;
+    const uint64_t begin = lo + lane < nseg ? segs[lo + lane].granule_begin : UINT64_MAX;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1)
+      if (__shfl_sync(0xFFFFFFFFu, begin, s + step) <= mine) s += step;
+    s += lo;
+  }
+  UnitRef<Io> r = unit_ref<Io>(segs[s], Io::kScaled ? inv_scale[s] : 1.0f, unit);
+  if (granule > last) r.rem = 0;
+  wait_for_previous();
+  axpy_unit<Io, Mode>(r, a);
+  let_next_start();
+}
+
 // The same with the segment table in the launch's parameters, for a caller without a
 // plan: no copy goes ahead of the kernel in its stream.
 template <class Io, class Mode>
@@ -1329,6 +1372,11 @@ cudaError_t launch_axpy_io(const PlanView& plan, const AxpyArgs& a, cudaStream_t
   auto k = axpy_noise_kernel<Io, Mode>;
   const Launch l = make_launch(reinterpret_cast<const void*>(k), axpy_shape<Io, Mode>().threads,
                                axpy_tile_units<Io, Mode>(), plan.granules);
+  if constexpr (!Mode::sum)
+    if (l.split.per_cta * kUnitsPerGranule <= static_cast<uint64_t>(l.block) &&
+        (plan.nseg > 1 || plan.granules <= kRowGranules))
+      return launch_early(axpy_row_kernel<Io, Mode>, l.grid, l.block, plan.early, stream, plan.segs,
+                          plan.nseg, plan.inv_scale, l.split, a);
   return launch_early(k, l.grid, l.block, plan.early, stream, plan.segs, plan.nseg, plan.inv_scale,
                       l.split, a);
 }

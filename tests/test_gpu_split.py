@@ -30,6 +30,45 @@ def test_segment_search(es, oracle, nseg):
     plan.close()
 
 
+# Passes whose CTAs have one row each, against the same tensors in a plan that a
+# further, larger one takes out of that range, bit for bit: tables of one to three
+# search steps, units at a segment's last elements, the high counter word changing
+# inside the set, the largest set of one segment and the next one.
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "fp8"])
+@pytest.mark.parametrize("nseg,total", [(1, 1), (1, 131_072), (1, 131_073), (2, 40), (3, 7_000),
+                                        (31, 5_000), (32, 90_000), (33, 300),
+                                        (40, 1_200_000), (1025, 40_000), (1100, 1_100_000)])
+def test_one_row_passes(es, dtype, nseg, total):
+    rng = np.random.default_rng(nseg + total)
+    numels = [int(n) for n in rng.integers(1, max(2, 2 * total // nseg), size=nseg)]
+    if nseg == 1:
+        numels = [total]
+    bases = [2**34 - 8 * (sum(numels) // 16)]
+    for n in numels[:-1]:
+        bases.append((bases[-1] + n + 7) // 8 * 8 + 8 * int(rng.integers(0, 3)))
+    if dtype == "fp8":
+        tensors = [torch.from_numpy(rng.integers(0, 120, size=n).astype(np.uint8)).cuda()
+                   for n in numels]
+        scales = [2.0**-9 * (1 + k % 5) for k in range(nseg)]
+    else:
+        tensors, scales = make_params(dtype, numels, seed=7), None
+    more = torch.zeros(1 << 22, dtype=tensors[0].dtype, device="cuda")
+    twins = [t.clone() for t in tensors]
+    small = es.plan_from_tensors(tensors, bases, scales)
+    large = es.plan_from_tensors(twins + [more], bases + [2**40], scales and scales + [1.0])
+    for what in ("es_perturb", "es_restore_perturb", "flip"):
+        for p in (small, large):
+            if what == "es_perturb":
+                es.es_perturb(p, 2**40 + 3, 1e-3)
+            else:
+                es.es_restore_perturb(p, 9, 1e-3, 9 if what == "flip" else 2**63, -1e-3)
+        torch.cuda.synchronize()
+        for x, y in zip(tensors, twins):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8)), what
+    small.close()
+    large.close()
+
+
 # One segment long enough for runs of whole tiles and rows in every CTA, the
 # high counter word changing inside it, against the same memory as many short
 # segments (units found one by one): bit-identical everywhere, and equal to the
