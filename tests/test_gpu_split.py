@@ -250,6 +250,172 @@ def test_launches_behind_other_work(es, numel):
     plan.close()
 
 
+# The same for every kernel that waits, in every storage type: the passes of one row,
+# of runs and of several segments, sums alone and with a perturb, the seed loop in one
+# generation, with a perturb and in several, the small sets' update, the fills and
+# (eager only: a capture refuses them) es_perturb_noalloc's short and long tables.
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "fp8"])
+@pytest.mark.parametrize("numel", [1000, 1 << 16, 3_000_001])
+def test_every_kernel_behind_other_work(es, dtype, numel):
+    torch.manual_seed(numel)
+    values = torch.empty(3, numel, device="cuda").normal_(0.0, 0.02)
+    scales = None
+    if dtype == "bf16":
+        values = values.to(torch.bfloat16)
+    elif dtype == "fp8":
+        values = (values * 2.0**9).to(torch.float8_e4m3fn).view(torch.uint8)
+        scales = [2.0**-9]
+    start, source, host = values[0].clone(), values[1].clone(), values[2].cpu().pin_memory()
+    a = start.clone()
+    # the same parameters as pieces of at least 16 elements
+    step = max(16, numel // 70 // 16 * 16)
+    bases = list(range(0, numel, step))
+    pieces = [a[o:o + step] for o in bases]
+    plan = es.plan_from_tensors([a], [0], scales)
+    cut = es.plan_from_tensors(pieces, bases, scales and scales * len(pieces))
+    segs = es.segments_from_tensors(pieces, bases)
+    raw = {"f32": es.ES_FP32, "bf16": es.ES_BF16}.get(dtype)
+    noise = torch.empty(numel, device="cuda")
+    other = torch.empty(numel, device="cuda")
+    seeds = np.arange(140, dtype=np.uint64) + 2**33
+    coeffs = np.linspace(1e-3, 2e-3, 140).astype(np.float32)
+    side = torch.cuda.Stream()
+
+    def add(x):
+        # another kernel that reads and writes the parameters
+        if dtype == "fp8":
+            a.bitwise_xor_(x & 1)
+        else:
+            a.add_(x)
+
+    def fork():
+        here = torch.cuda.current_stream()
+        side.wait_stream(here)
+        with torch.cuda.stream(side):
+            es.es_noise_fill(6, 0, numel, other)
+        add(source)
+        here.wait_stream(side)
+
+    def fill():
+        es.es_noise_fill(5, 3, numel, a if dtype == "f32" else noise)
+        if dtype != "f32":
+            a.copy_(noise if dtype == "bf16" else source)
+
+    calls_ = [
+        lambda p: es.es_perturb(p, 3, 1e-3),
+        lambda p: es.es_restore_perturb(p, 3, 1e-3, 4, 1e-3),
+        lambda p: es.es_restore_perturb(p, 4, 1e-3, 4, -1e-3),
+        lambda p: es.es_update(p, seeds[:6], coeffs[:6]),
+        lambda p: es.es_update(p, seeds[:2], coeffs[:2]),
+        lambda p: es.es_update_perturb(p, seeds[:2], coeffs[:2], 9, 1e-3),
+        lambda p: es.es_update(p, seeds[:9], coeffs[:9]),
+        lambda p: es.es_update(p, seeds[:129], coeffs[:129]),
+        lambda p: es.es_update_perturb(p, seeds[:12], coeffs[:12], 9, 1e-3),
+        lambda p: es.es_replay(p, seeds[:17], coeffs[:17], [2, 9, 1, 5]),
+        lambda p: es.es_replay(p, seeds, coeffs, [70, 1, 69]),
+    ]
+    unplanned = [lambda: es.es_perturb_noalloc(segs[:40], raw, 8, 1e-3),
+                 lambda: es.es_perturb_noalloc(segs, raw, 8, 1e-3)]
+
+    def calls(wait, eager):
+        out = []
+        for before in (lambda: a.copy_(start), lambda: a.copy_(host, non_blocking=True),
+                       lambda: a.zero_(), lambda: add(source), fill, fork):
+            before()
+            wait()
+            for p in (plan, cut):
+                for call in calls_:
+                    call(p)
+                    wait()
+            for call in unplanned if eager and raw is not None else ():
+                call()
+                wait()
+            out.append(a.clone())
+            wait()
+        return out
+
+    def same(want, got):
+        torch.cuda.synchronize()
+        for x, y in zip(want, got):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+
+    want = calls(torch.cuda.synchronize, True)
+    for _ in range(2):
+        a.copy_(start)
+        same(want, calls(lambda: None, True))
+    a.copy_(start)
+    want = calls(torch.cuda.synchronize, False)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = calls(lambda: None, False)
+    for _ in range(2):
+        graph.replay()
+        same(want, got)
+    plan.close()
+    cut.close()
+
+
+# A kernel of another library behind a launch does not start early: it reads what the
+# launch has written (es_noise_fill's buffer and an updated set, summed).
+@pytest.mark.parametrize("numel", [1000, 1 << 16, 3_000_001])
+def test_other_work_behind_launches(es, numel):
+    a = torch.zeros(numel, device="cuda")
+    plan = es.plan_from_tensors([a])
+    out = torch.zeros(numel, device="cuda")
+    seeds, coeffs = np.arange(9, dtype=np.uint64), np.full(9, 1e-3, dtype=np.float32)
+
+    def calls(wait):
+        got = []
+        for call in (lambda: es.es_perturb(plan, 3, 1.0), lambda: es.es_update(plan, seeds, coeffs),
+                     lambda: es.es_update(plan, seeds[:2], coeffs[:2]),
+                     lambda: es.es_noise_fill(7, 1, numel, out)):
+            a.zero_()
+            out.zero_()
+            wait()
+            call()
+            wait()
+            got.append(a + out)
+            wait()
+        return got
+
+    want = calls(torch.cuda.synchronize)
+    for _ in range(3):
+        got = calls(lambda: None)
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(want, got))
+    plan.close()
+
+
+# es_perturb_noalloc calls of up to 64 segments share nothing: on two streams at once,
+# with different tables, each gives what its plan gives.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_short_tables_on_two_streams(es, dtype):
+    kind = es.ES_BF16 if dtype == "bf16" else es.ES_FP32
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    sets, twins, tables, plans = [], [], [], []
+    for k, nseg in enumerate((64, 37)):
+        tensors = make_params(dtype, [3_000 + 977 * i for i in range(nseg)], seed=k)
+        twin = [t.clone() for t in tensors]
+        plan, segs = build_plan(es, twin)
+        sets.append(tensors)
+        twins.append(twin)
+        tables.append(es.segments_from_tensors(tensors, [s.index_base for s in segs]))
+        plans.append(plan)
+    torch.cuda.synchronize()
+    for i in range(25):
+        for k in (0, 1):
+            es.es_perturb_noalloc(tables[k], kind, 100 * k + i, 1e-3, stream=streams[k])
+    torch.cuda.synchronize()
+    for i in range(25):
+        for k in (0, 1):
+            es.es_perturb(plans[k], 100 * k + i, 1e-3)
+    torch.cuda.synchronize()
+    for tensors, twin, plan in zip(sets, twins, plans):
+        for x, y in zip(tensors, twin):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+        plan.close()
+
+
 # A plan is ready on every stream when it is handed out: used at once on a stream
 # that does not synchronise with the default one and is still busy, its table (and
 # FP8's scales) are those of the same call on a plan made long before.
