@@ -358,7 +358,7 @@ es_status_t es_fold_antithetic(const double* rhat_pos, const double* rhat_neg,
  * itself; a longer one is copied (cudaMemcpyAsync on `stream`) into one static
  * device array of ES_STATIC_MAX_SEGMENTS + 1 descriptors (about 32 KB), which every
  * device that loads the library holds until the process exits. The entry point
- * calls no cudaMalloc, cudaFree or other allocating routine, and uses about 38 KB
+ * calls no cudaMalloc, cudaFree or other allocating routine, and uses about 44 KB
  * of host stack.
  *   - More than ES_STATIC_MAX_SEGMENTS segments: ES_ERR_INVALID_ARG, nothing
  *     is launched.

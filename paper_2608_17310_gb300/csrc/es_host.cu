@@ -438,8 +438,14 @@ es_status_t es_replay(es_plan_t plan, const uint64_t* seeds, const float* coeffs
   // parameters on a generation gets a pass of its own, through the
   // single-generation kernels, which run faster than the shared pass's rounding
   // between generations. Not so one fp32 seed, bound by HBM alone. Measured, us
-  // for 8 generations, shared / own: 2 bf16 seeds over 2^20 parameters 16.5 / 31.0,
-  // 2^24 203 / 217, 2^26 800 / 785, 2^28 3181 / 2993; 1 fp32 seed 2^28 1686 / 2629.
+  // for 8 generations, shared / own: 2 bf16 seeds over 2^20 parameters 15.6 / 23.5,
+  // 2^22 52.5 / 64.9, 2^24 201.5 / 202.2, 2^25 400 / 383, 2^26 798 / 750; 8 bf16 seeds
+  // 52.2 / 67.0, 189 / 199, 745 / 730, 1487 / 1443, 2971 / 2865; 1 fp32 seed 2^26
+  // 425 / 670. The line is one for every population and type, and sharing costs some
+  // of them a little below it: up to 16 seeds at most 4.5 % (8 FP8 seeds over 2^24
+  // 758 / 725), 64 seeds 2 to 13 % (fp32 2^24 6135 / 5706, 2^18 143 / 127), or 27 %
+  // where each generation by itself would take the small sets' kernel but all of them
+  // hold more than its 128 seeds (fp32 65,536 parameters 108 / 86).
   constexpr uint64_t kOwnPass = uint64_t{1} << 25;
   const bool large = plan->numel >= kOwnPass;
   const int own_from = plan->dtype == ES_FP32 ? 2 : 1;

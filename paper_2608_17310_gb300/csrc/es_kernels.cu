@@ -488,6 +488,10 @@ struct AxpyGens {
 // 1088 / 1579 / 2115 / 4171; with the perturb behind 1 / 4 / 8 bf16 seeds 1656 / 3249 / 5433
 // -> 1107 / 2675 / 4752. 12 and 16 seeds unrolled gain 3 and 1 % on the loop, for twice
 // the code: not built.
+// fp32: 4 vectors, 2 ahead, while HBM bounds the pass (perturb 958, against 1133 with
+// one vector) and as far as that body fits into 64 registers with few spills (4
+// schedules 2167 against 2182, with 220 bytes spilled; 896 threads 2161, 768 2213); from
+// 5 on one vector (5 schedules 2858 -> 2745, 8 6243 -> 4354).
 // Thread counts that are no multiple of 128 leave the SM's four schedulers
 // unequal warps and run 10 % slower.
 struct AxpyShape {
@@ -527,9 +531,9 @@ __device__ __forceinline__ void axpy_run(typename Io::Scalar* p, uint64_t j_thre
   constexpr int D = kShape.ahead;
   constexpr int kStride = kShape.threads * V;  // elements between a thread's vectors
   static_assert(kShape.vecs % D == 0, "the vectors in flight rotate within a tile");
-  // the one-seed pass is fastest with every Philox product 64-bit wide (in
-  // FP8 storage, with twice the blocks per vector, that spills)
-  constexpr bool kWide = Mode::kind == AxpyKind::kSteps && Mode::seeds == 1 && V <= 8;
+  // the one-seed pass is fastest with every Philox product 64-bit wide (FP8, the
+  // least of the three: 572.7 -> 570.6 us over 792,680,960 parameters)
+  constexpr bool kWide = Mode::kind == AxpyKind::kSteps && Mode::seeds == 1;
   const uint32_t j_hi = static_cast<uint32_t>(j_thread >> 32);
   const AxpyGens<Mode, kWide> gens(a, j_hi);
   Round0 p0 = philox_round0<kWide>(static_cast<uint32_t>(j_thread));
@@ -627,8 +631,11 @@ __device__ __forceinline__ void axpy_pass(const SegDesc* __restrict__ segs, int 
     const int last = search_segment(segs, seg, nseg, (stop - 1) / kUnitsPerGranule);
     wait_for_previous();
     // Units of one segment take its entry from registers, which saves a launch
-    // 0.2-0.5 us (2^22 bf16 parameters 5.9 -> 5.5 us); in the bf16 two-step pass
-    // and sums the second loop costs the run above 2 % instead
+    // 0.2-0.5 us (2^22 bf16 parameters 5.9 -> 5.5 us). Not in the two-step pass and
+    // the sums of the 8-element types, bf16 and FP8, where the second loop costs the
+    // run above: bf16 2 %; FP8 over 792,680,960 parameters two steps 1118 -> 1126 us,
+    // 4 seeds 2116 -> 2126, while launches over 2^18 to 2^22 parameters would gain
+    // 0.1-0.4 us with 1 or 2 seeds and lose 0.1-0.2 with 4 or more
     constexpr bool kKeep = Io::kVec != 8 || (!Mode::sum && Mode::seeds == 1);
     bool done = false;
     if constexpr (kKeep) {
@@ -880,12 +887,16 @@ __device__ __forceinline__ void update_unit(typename Io::Scalar* p, int rem, flo
 // one segment from a pointer and a counter that are stepped, and
 // single rows, each thread finding its own segment, where a segment, the range
 // or a high counter word ends.
-// Bound by the generator like the passes above. Measured over 792,680,960
-// parameters (ms; 3 CTAs of 256 threads on grid-stride tiles -> one CTA of 640):
-// 8 seeds bf16 4.70 -> 4.43 (1.43e12 Gaussians/s), fp32 5.32 -> 4.42 and FP8
-// 4.90 -> 4.41 (their seed loops were not pipelined: they took 8 elements in another form), 16 seeds +
-// perturb bf16 9.77 -> 9.15. Several generations run fastest
-// with 768: 8 generations of 2 seeds 10.59 -> 9.41.
+// What comes here: one generation of more than 8 seeds, and the passes that several
+// generations of a replay share (es_replay), both where update_split_kernel does not
+// take them.
+// Bound by the generator like the passes above. Measured (3 CTAs of 256 threads on
+// grid-stride tiles -> one CTA of 640), ms over 792,680,960 parameters: 16 seeds bf16
+// 8.99 -> 8.59 (1.48e12 Gaussians/s), fp32 10.24 -> 8.55 and FP8 9.61 -> 8.59 (their
+// seed loops were not pipelined: they took 8 elements in another form), 128 seeds bf16
+// 69.0 -> 67.1, 16 seeds + perturb bf16 9.77 -> 9.16. Several generations take 768
+// threads, us over 2^24 parameters for 8 generations of 2 seeds (as before; 640 -> 768):
+// bf16 228; 205.7 -> 201.8, FP8 236; 206.6 -> 207.0, but fp32 243; 200.4 -> 203.8.
 template <bool kSingle>
 __host__ __device__ constexpr int update_threads() {
   return kSingle ? 640 : 768;
@@ -968,14 +979,22 @@ update_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __restric
 // element of a block, which add them up in ascending seed order with the same
 // operations as update_unit, so the values are the same bits. What bounds it is
 // latency: n / kWarps rounds of one block's generation instead of n of two blocks'.
-// 65,536 fp32 parameters, us in a graph (the seed loop's or the sums' pass -> this):
-// 1 seed 1.7 -> 1.6, 8 seeds 3.0 -> 2.1, 32 seeds 6.9 -> 5.8, 128 seeds 21.9 -> 20.0;
-// 1024 parameters 32 seeds 6.8 -> 2.5. It generates one block per thread where
-// update_unit overlaps two, so it loses once the GPU is full: 98,304 parameters, 8
-// seeds even, 128 seeds 22.2 -> 29.5. kSplitMaxGranules lies where 128 seeds break
-// even. A CTA of 32 warps, 32 seeds at a time, is the better one while every CTA
-// has an SM to itself (19,000 parameters, 128 seeds 12.6 with 8 warps -> 9.2; 65,536: 20.4 ->
-// 24.0).
+// fp32, us in a graph (the sums' pass or the seed loop -> this): 1,024 parameters 1 seed
+// 1.36 -> 1.12, 32 seeds 6.6 -> 2.4, 128 seeds 22.5 -> 8.6; 65,536 parameters 1.53 ->
+// 1.57, 7.0 -> 6.0, 22.4 -> 20.5, and 8 seeds 2.9 -> 2.2. It generates one block per
+// thread where the others overlap two, so it loses once the GPU is full, at a size that
+// depends on the population: 1 and 2 seeds are even at 65,536 parameters, 8 seeds at
+// 98,304 (2.9 -> 2.8), 16 and 32 at 81,920 (7.1 -> 7.2); 128 seeds gain there yet (30.3,
+// where the loop's rows just miss its CTAs, -> 25.2) and lose at 98,304 (22.4 -> 29.7).
+// kSplitMaxGranules, 69,632 parameters, is one line for all: up to it only 1 seed loses,
+// 0.06 us (bf16 0.11), and 32 gain 7.1 -> 6.0, 128 22.3 -> 20.5.
+// A launch of more than kSplitSeeds seeds does not come here whatever its size. That
+// is what SplitArgs holds and no break-even: 129 seeds take the seed loop 23.3 us over
+// 1,000 parameters, where 128 take 8.7, and 22.8 against 20.5 over 65,536.
+// A CTA of 32 warps, 32 seeds at a time, is taken for more than 8 while every CTA has
+// one of the GPU's 152 SMs to itself (19,456 parameters, 128 seeds 13.1 with 8 warps ->
+// 9.1). With two on an SM it still gains from 32 seeds on (32,768 parameters 13.7 ->
+// 12.2) and loses with 16 (2.59 -> 2.63); at 65,536 it loses with any (20.5 -> 23.8).
 constexpr uint64_t kSplitMaxGranules = 4352;
 constexpr uint64_t kSplitWideGranules = 152 * 8;
 constexpr int kSplitSeeds = 128;
@@ -1072,9 +1091,9 @@ update_split_kernel(const SegDesc* __restrict__ segs, int nseg, const float* __r
 // once and every store is a coalesced 16 bytes. Only the first and the last
 // group, which may reach beyond [0, n), store element by element.
 // Bound by the generator, and by the stores' bandwidth not far behind (500,000,000
-// aligned floats run at 5.9 TB/s). 50,000,003 floats from an unaligned index 58.8 us
-// (4-byte stores, every block through the general rounds) -> 40.7; 50,000,000
-// aligned 43.8 (256-thread CTAs, one block at a time) -> 36.7, 500,000,000 418 -> 347.
+// aligned floats run at 5.76 TB/s). 50,000,003 floats from an unaligned index 58.4 us
+// (4-byte stores, every block through the general rounds) -> 40.3; 50,000,000
+// aligned 44.3 (256-thread CTAs, one block at a time) -> 36.8, 500,000,000 418 -> 347.
 // 512 to 768 threads and 2 pairs of rows per loop are within 2 %; 1024 threads lose 8 %.
 struct FillArgs {
   PhiloxSched sched;
