@@ -58,10 +58,11 @@ class EsError(RuntimeError):
 
 
 _lib = None
+_address_calls = None
 
 
 def _load() -> ctypes.CDLL:
-    global _lib
+    global _lib, _address_calls
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -104,20 +105,27 @@ def _load() -> ctypes.CDLL:
     # small calls are bound by their host time (es_update of a set that one SM holds:
     # 14.5 us a call with typed pointers and a Stream object, 6.2 us so). L[name] is a
     # function object of its own, so a caller of lib() keeps the typed ones.
-    L.by_address = SimpleNamespace()
+    by_address = SimpleNamespace()
     for name in ("es_update", "es_update_perturb", "es_replay", "es_normalize_rewards",
                  "es_update_coeffs", "es_fold_antithetic"):
         res, args = sigs[name]
         fn = L[name]
         fn.restype = res
         fn.argtypes = [vp if a in (P(u64), P(f32), P(f64), P(i32)) else a for a in args]
-        setattr(L.by_address, name, fn)
+        setattr(by_address, name, fn)
+    _address_calls = by_address
     _lib = L
     return L
 
 
 def lib() -> ctypes.CDLL:
     return _load()
+
+
+def _by_address() -> SimpleNamespace:
+    if _lib is None:
+        _load()
+    return _address_calls
 
 
 def _status_string(status: int) -> str:
@@ -324,8 +332,8 @@ def es_update(plan: Plan, seeds, coeffs, stream=None) -> None:
     c = np.ascontiguousarray(coeffs, dtype=np.float32)
     if s.size != c.size:
         raise ValueError("seeds and coeffs differ in length")
-    _check(_load().by_address.es_update(plan.handle, _addr(s), _addr(c), s.size,
-                                        _stream(stream)), "es_update")
+    _check(_by_address().es_update(plan.handle, _addr(s), _addr(c), s.size, _stream(stream)),
+           "es_update")
 
 
 def es_perturb_noalloc(segments: Sequence[Segment], dtype: int, seed: int, sigma: float,
@@ -344,9 +352,8 @@ def es_update_perturb(plan: Plan, seeds, coeffs, next_seed: int, sigma_next: flo
     c = np.ascontiguousarray(coeffs, dtype=np.float32)
     if s.size != c.size:
         raise ValueError("seeds and coeffs differ in length")
-    _check(_load().by_address.es_update_perturb(plan.handle, _addr(s), _addr(c), s.size, next_seed,
-                                                sigma_next, _stream(stream)),
-           "es_update_perturb")
+    _check(_by_address().es_update_perturb(plan.handle, _addr(s), _addr(c), s.size, next_seed,
+                                           sigma_next, _stream(stream)), "es_update_perturb")
 
 
 def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
@@ -356,8 +363,8 @@ def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
     n = np.ascontiguousarray(counts, dtype=np.int32)
     if s.size != c.size or int(n.sum()) != s.size:
         raise ValueError("seeds, coeffs and counts do not agree")
-    _check(_load().by_address.es_replay(plan.handle, _addr(s), _addr(c), _addr(n), n.size,
-                                        _stream(stream)), "es_replay")
+    _check(_by_address().es_replay(plan.handle, _addr(s), _addr(c), _addr(n), n.size,
+                                   _stream(stream)), "es_replay")
 
 
 # --- host-side generation control ---------------------------------------------------
@@ -365,7 +372,7 @@ def es_replay(plan: Plan, seeds, coeffs, counts, stream=None) -> None:
 def es_normalize_rewards(rewards, eps_z: float = 1e-8) -> np.ndarray:
     r = _f64(rewards)
     out = np.empty_like(r)
-    _check(_load().by_address.es_normalize_rewards(_addr(r), r.size, eps_z, _addr(out)),
+    _check(_by_address().es_normalize_rewards(_addr(r), r.size, eps_z, _addr(out)),
            "es_normalize_rewards")
     return out
 
@@ -377,7 +384,7 @@ def es_sigma_cosine(sigma0: float, sigmaT: float, t: int, T: int) -> float:
 def es_update_coeffs(rhat, alpha: float, sigma: float, mode: int = ES_SCALE_PAPER) -> np.ndarray:
     r = _f64(rhat)
     out = np.empty(r.size, dtype=np.float32)
-    _check(_load().by_address.es_update_coeffs(_addr(r), r.size, alpha, sigma, mode, _addr(out)),
+    _check(_by_address().es_update_coeffs(_addr(r), r.size, alpha, sigma, mode, _addr(out)),
            "es_update_coeffs")
     return out
 
@@ -388,6 +395,6 @@ def es_fold_antithetic(rhat_pos, rhat_neg, alpha: float, sigma: float,
     if p.size != m.size:
         raise ValueError("rhat_pos and rhat_neg differ in length")
     out = np.empty(p.size, dtype=np.float32)
-    _check(_load().by_address.es_fold_antithetic(_addr(p), _addr(m), p.size, alpha, sigma, mode,
-                                                 _addr(out)), "es_fold_antithetic")
+    _check(_by_address().es_fold_antithetic(_addr(p), _addr(m), p.size, alpha, sigma, mode,
+                                            _addr(out)), "es_fold_antithetic")
     return out
